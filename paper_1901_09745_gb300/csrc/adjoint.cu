@@ -79,7 +79,7 @@ k_adjoint(const T *__restrict__ gt, const T *__restrict__ lam_in, T *__restrict_
     const T uF = u[0] * F[0] + u[1] * F[1] + u[2] * F[2];
 
     // ---- the cell's total solid fraction and weight (Table 1, Eq. 9 at eps_n)
-    const T cx = (T)threadIdx.x, cy = (T)threadIdx.y, cz = (T)threadIdx.z;
+    const T cx = (T)((int)threadIdx.x - L::REC_X), cy = (T)threadIdx.y, cz = (T)threadIdx.z;
     T seps = 0;
     if (cnt > 0) {
         __syncthreads();
@@ -287,11 +287,11 @@ cudaError_t launch_adjoint(int storage, int lattice, const void *gt, const void 
                            const Geom &g, const Phys &ph, const Tiles &tl, const Parts &pd, double invT,
                            double *dJdX, double *dFpart, cudaStream_t s) {
     if (storage == ST_F64) {
-        return lattice == 9 ? launch_adjoint_t<D2Q9, double>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s)
-                            : launch_adjoint_t<D3Q19, double>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
+        return lattice == 9 ? launch_adjoint_t<Tiled<D2Q9, double>, double>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s)
+                            : launch_adjoint_t<Tiled<D3Q19, double>, double>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
     }
-    return lattice == 9 ? launch_adjoint_t<D2Q9, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s)
-                        : launch_adjoint_t<D3Q19, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
+    return lattice == 9 ? launch_adjoint_t<Tiled<D2Q9, float>, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s)
+                        : launch_adjoint_t<Tiled<D3Q19, float>, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
 }
 
 }  // namespace psc
@@ -454,6 +454,7 @@ extern "C" lbm_status lbm_adjoint_backward(lbm_ctx *ctx, long long token, double
         const double invT = 1.0 / nsteps;
         tl.count = ctx->tile_count; tl.list = ctx->tile_list; tl.cap = ctx->p.tile_cap;
         tl.stats = ctx->tile_stats; tl.blocks = ctx->tile_blocks; tl.order = ctx->tile_order;
+        tl.work = ctx->step_work;
         scratch_parts = ctx_parts(ctx);
         scratch_parts.F = w.sF;
         scratch_parts.T = w.sT;

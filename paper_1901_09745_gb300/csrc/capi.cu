@@ -208,7 +208,7 @@ extern "C" lbm_status lbm_create(const lbm_params *p, lbm_ctx **out) {
         set_face_kind(g, a, 1, lo == FACE_INFLOW ? FACE_OUTLET : lo);
     }
     for (int a = 0; a < 3; ++a) {
-        g.nt[a] = (g.n[a] + tile_ext(ctx->dim, a) - 1) / tile_ext(ctx->dim, a);
+        g.nt[a] = (g.n[a] + tile_ext(ctx->dim, wide_tiles(ctx->dim, ctx->elem, ctx->g), a) - 1) / tile_ext(ctx->dim, wide_tiles(ctx->dim, ctx->elem, ctx->g), a);
         g.inv_n[a] = 1.0 / g.n[a];
     }
     ctx->ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
@@ -241,6 +241,8 @@ extern "C" lbm_status lbm_create(const lbm_params *p, lbm_ctx **out) {
     if (e == cudaSuccess) e = cudaMalloc(&ctx->f[0], bytes);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->f[1], bytes);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->flags, 4 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->step_work, kWorkWords * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->step_work, 0, kWorkWords * sizeof(int), ctx->stream);
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&ctx->hflags, 4 * sizeof(int), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&ctx->hflags_dev, ctx->hflags, 0);
     // rest state f_i = w_i: every stored deviation is zero (all-zero bits in every format)
@@ -264,6 +266,7 @@ extern "C" lbm_status lbm_destroy(lbm_ctx *ctx) {
     if (ctx->dem) dem_release(ctx->dem);
     free_dev(&ctx->f[0]); free_dev(&ctx->f[1]);
     free_dev((void **)&ctx->flags);
+    free_dev((void **)&ctx->step_work);
     if (ctx->hflags) cudaFreeHost(ctx->hflags);
     free(ctx->hR);
     for (int k = 0; k < 2; ++k) {
@@ -305,6 +308,7 @@ static Tiles ctx_tiles(lbm_ctx *ctx) {
     tl.count = ctx->tile_count; tl.list = ctx->tile_list; tl.cap = ctx->p.tile_cap; tl.stats = ctx->tile_stats;
     tl.order = ctx->tile_order;
     tl.blocks = ctx->tile_blocks;
+    tl.work = ctx->step_work;
     return tl;
 }
 
@@ -312,7 +316,7 @@ static Tiles ctx_tiles(lbm_ctx *ctx) {
 // the widest particle shell does not fit well inside half the box.
 void ctx_update_wrap(lbm_ctx *ctx) {
     for (int a = 0; a < 3; ++a) {
-        double need = tile_ext(ctx->dim, a) + 2.0 * (ctx->rmax + ctx->p.shell_h) + 2.0;
+        double need = tile_ext(ctx->dim, wide_tiles(ctx->dim, ctx->elem, ctx->g), a) + 2.0 * (ctx->rmax + ctx->p.shell_h) + 2.0;
         const int w = (a < ctx->dim && ctx->g.periodic[a] && ctx->g.n[a] < need) ? 1 : 0;
         if (w != ctx->g.wrap_img[a]) ctx->gen += 1;     // the step's kernels take Geom by value
         ctx->g.wrap_img[a] = w;
@@ -369,7 +373,7 @@ static lbm_status ctx_reserve_tiles(lbm_ctx *ctx) {
     CK(cudaMalloc(&ctx->tile_count, (size_t)ctx->ntiles * sizeof(int)), "cudaMalloc(tile counts)");
     CK(cudaMalloc(&ctx->tile_list, (size_t)ctx->ntiles * ctx->p.tile_cap * sizeof(int)), "cudaMalloc(tile lists)");
     CK(cudaMalloc(&ctx->tile_stats, kTileStats * sizeof(int)), "cudaMalloc(tile stats)");
-    CK(cudaMalloc(&ctx->tile_order, (size_t)ctx->ntiles * 3 * sizeof(uint2)), "cudaMalloc(tile order)");
+    CK(cudaMalloc(&ctx->tile_order, (size_t)ctx->ntiles * 3 * sizeof(unsigned)), "cudaMalloc(tile order)");
     CK(cudaMalloc(&ctx->tile_blocks, (size_t)ctx->ntiles * pack_block_bytes(ctx->p.storage == LBM_F64, ctx->p.tile_cap)),
        "cudaMalloc(tile candidate blocks)");
     CK(cudaMemsetAsync(ctx->tile_stats, 0, kTileStats * sizeof(int), ctx->stream), "memset tile stats");
@@ -549,8 +553,8 @@ static lbm_status ctx_enqueue_bin(lbm_ctx *ctx) {
     Tiles tl = ctx_tiles(ctx);
     CK(cudaMemsetAsync(ctx->tile_count, 0, (size_t)ctx->ntiles * sizeof(int), ctx->stream), "memset tile counts");
     CK(cudaMemsetAsync(ctx->tile_stats, 0, kTileStats * sizeof(int), ctx->stream), "memset tile stats");
-    CK(launch_bin(ctx->dim, ctx->g, ctx->ph, tl, ctx_parts(ctx), ctx->stream), "bin kernel");
-    CK(launch_pack(ctx->q, ctx->p.storage == LBM_F64, ctx->g, tl, ctx_parts(ctx), ctx->ntiles, ctx->stream), "pack kernel");
+    CK(launch_bin(ctx->dim, wide_tiles(ctx->dim, ctx->elem, ctx->g), ctx->g, ctx->ph, tl, ctx_parts(ctx), ctx->stream), "bin kernel");
+    CK(launch_pack(ctx->q, ctx->p.storage, ctx->g, tl, ctx_parts(ctx), ctx->ntiles, ctx->stream), "pack kernel");
     return LBM_OK;
 }
 
@@ -636,8 +640,7 @@ lbm_status ctx_step_once(lbm_ctx *ctx) {
         ctx->launches += 2;
         ctx->bins_valid = 1;
     }
-    // all tiles (2D: particle and fluid tiles), overflow tiles
-    ctx->launches += (ctx->np > 0) ? ((ctx->q == 9 && ctx->p.storage != LBM_F64) ? 3 : 2) : 1;
+    ctx->launches += (ctx->np > 0) ? 2 : 1;     // the step's kernel, the overflow tiles
     ctx->cs_launches += 1;
     ctx->cur ^= 1;
     ctx->steps += 1;

@@ -41,7 +41,8 @@ struct lbm_ctx {
     // tile candidate lists
     long long ntiles;
     int *tile_count, *tile_list, *tile_stats;
-    uint2 *tile_order;
+    unsigned *tile_order;
+    int *step_work;            // work counters of the step's kernel (see Tiles)
     void *tile_blocks;         // packed candidate records per tile
     int bins_valid;
 

@@ -95,10 +95,11 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
         // radii are device data here, so every periodic axis takes the per-cell minimum image
         // (always exact; only the cost of a few extra instructions)
         g.wrap_img[a] = (a < (is2d ? 2 : 3)) && g.periodic[a];
-        g.nt[a] = (g.n[a] + tile_ext(is2d ? 2 : 3, a) - 1) / tile_ext(is2d ? 2 : 3, a);
         g.inv_n[a] = 1.0 / g.n[a];
     }
-    if (g.nt[1] > 65535 || g.nt[2] > 65535) return fail(LBM_ERR_ARG, "ny or nz too large for the tile grid");
+    const int wide = wide_tiles(is2d ? 2 : 3, elem, g);
+    for (int a = 0; a < 3; ++a) g.nt[a] = (g.n[a] + tile_ext(is2d ? 2 : 3, wide, a) - 1) / tile_ext(is2d ? 2 : 3, wide, a);
+    if ((g.n[1] + tile_ext(is2d ? 2 : 3, 0, 1) - 1) / tile_ext(is2d ? 2 : 3, 0, 1) > 65535 || g.nt[2] > 65535) return fail(LBM_ERR_ARG, "ny or nz too large for the tile grid");
     Phys ph;
     ph.tau = p->tau;
     for (int a = 0; a < 3; ++a) ph.body_force[a] = p->body_force[a];
@@ -111,16 +112,17 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
     for (int a = 0; a < 3; ++a)
         if (p->bc[a] == LBM_BC_INFLOW) ph.inflow_axis = a;
 
-    // carve the fixed array: counts | stats | flags | lists | tile order | f(r) | packed tile blocks
+    // carve the fixed array: counts | stats | flags | work counters | lists | tile order | f(r) | packed tile blocks
     const long long ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
     const int rec_double = (p->storage == LBM_F64);
     size_t off = 0;
     const size_t o_count = off; off += (size_t)ntiles * sizeof(int);
     const size_t o_stats = off; off += kTileStats * sizeof(int);
     const size_t o_flags = off; off += 4 * sizeof(int);
+    const size_t o_work = off; off += kWorkWords * sizeof(int);
     const size_t o_list = off; off += (size_t)ntiles * kNoAllocCap * sizeof(int);
     off = align_up(off, 16);
-    const size_t o_order = off; off += (size_t)ntiles * 3 * sizeof(uint2);
+    const size_t o_order = off; off += (size_t)ntiles * 3 * sizeof(unsigned);
     off = align_up(off, 16);
     const size_t o_fr = off; off += (size_t)n * sizeof(double);
     off = align_up(off, 256);
@@ -161,18 +163,19 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
     tl.list = (int *)(base + o_list);
     tl.cap = kNoAllocCap;
     tl.blocks = base + o_blocks;
-    tl.order = (uint2 *)(base + o_order);
+    tl.order = (unsigned *)(base + o_order);
+    tl.work = (int *)(base + o_work);
     int *flags = (int *)(base + o_flags);
     Parts pd;
     pd.n = n; pd.X = X; pd.U = U; pd.Om = Omega; pd.R = radius; pd.Fr = (double *)(base + o_fr);
     pd.F = F; pd.T = T;
     pd.Pf = nullptr;
 
-    // what must start at zero: tile counts, stats, flags (the rest is fully rewritten)
+    // what must start at zero: tile counts, stats, flags, work counters (the rest is fully rewritten)
     e = cudaMemsetAsync(base, 0, o_list, s);
     if (e == cudaSuccess && n > 0) e = launch_f_of_r(is2d ? 2 : 3, radius, (double *)(base + o_fr), n, s);
-    if (e == cudaSuccess && n > 0) e = launch_bin(is2d ? 2 : 3, g, ph, tl, pd, s);
-    if (e == cudaSuccess && n > 0) e = launch_pack(p->lattice, rec_double, g, tl, pd, ntiles, s);
+    if (e == cudaSuccess && n > 0) e = launch_bin(is2d ? 2 : 3, wide, g, ph, tl, pd, s);
+    if (e == cudaSuccess && n > 0) e = launch_pack(p->lattice, p->storage, g, tl, pd, ntiles, s);
     if (e == cudaSuccess)
         e = launch_collide_stream(p->storage, p->lattice, f_in, f_out, g, ph, tl, pd, flags, s,
                                   g_overlap[dev].join ? &g_overlap[dev] : nullptr);

@@ -12,7 +12,7 @@ namespace psc {
 
 constexpr int kBinBatch = 8;   // tiles whose slot atomics one thread has in flight at once
 
-__global__ void k_bin(int dim, Geom g, double h, Tiles tl, Parts pd) {
+__global__ void k_bin(int dim, int wide, Geom g, double h, Tiles tl, Parts pd) {
     pdl_launch();     // the packing kernel may start; it waits for this one to finish
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     int mx = 0;   // largest slot taken by this thread
@@ -39,7 +39,7 @@ __global__ void k_bin(int dim, Geom g, double h, Tiles tl, Parts pd) {
             if (ax >= dim) { nr[ax] = 1; ra[ax][0] = rb[ax][0] = 0; len[ax] = 1; continue; }
             const double X = xw[ax];
             const int lo = (int)ceil(X - r - h), hi = (int)floor(X + r + h);
-            nr[ax] = axis_tile_ranges(lo, hi, g.n[ax], tile_ext(dim, ax), g.nt[ax], g.periodic[ax], ra[ax], rb[ax]);
+            nr[ax] = axis_tile_ranges(lo, hi, g.n[ax], tile_ext(dim, wide, ax), g.nt[ax], g.periodic[ax], ra[ax], rb[ax]);
             len[ax] = 0;
             for (int k = 0; k < nr[ax]; ++k) len[ax] += rb[ax][k] - ra[ax][k] + 1;
         }
@@ -58,8 +58,8 @@ __global__ void k_bin(int dim, Geom g, double h, Tiles tl, Parts pd) {
                     const int ty = axis_tile(kyz % len[1], nr[1], ra[1], rb[1]);
                     const int tz = axis_tile(kyz / len[1], nr[2], ra[2], rb[2]);
                     tile[q] = -1;
-                    const int org[3] = {tx * tile_ext(dim, 0), ty * tile_ext(dim, 1), tz * tile_ext(dim, 2)};
-                    const int ext[3] = {tile_ext(dim, 0), tile_ext(dim, 1), tile_ext(dim, 2)};
+                    const int org[3] = {tx * tile_ext(dim, wide, 0), ty * tile_ext(dim, wide, 1), tz * tile_ext(dim, wide, 2)};
+                    const int ext[3] = {tile_ext(dim, wide, 0), tile_ext(dim, wide, 1), tile_ext(dim, wide, 2)};
                     if (tile_in_reach(xp, reach, org, ext, g.n, g.periodic, dim)) {
                         tile[q] = PSC_IDX(tx + (long long)g.nt[0] * (ty + (long long)g.nt[1] * tz),
                                           (long long)g.nt[0] * g.nt[1] * g.nt[2], CHK_TILE);
@@ -142,11 +142,11 @@ __global__ void k_download(const double *F, const double *T, double *Fo, double 
     if (k < 4) flags_out[k] = flags[k];
 }
 
-cudaError_t launch_bin(int dim, const Geom &g, const Phys &ph, const Tiles &tl, const Parts &pd,
+cudaError_t launch_bin(int dim, int wide, const Geom &g, const Phys &ph, const Tiles &tl, const Parts &pd,
                        cudaStream_t s) {
     if (pd.n <= 0) return cudaSuccess;
     const int threads = 128;
-    return launch_pdl(k_bin, dim3((pd.n + threads - 1) / threads), dim3(threads), 0, s, dim, g, ph.shell_h, tl, pd);
+    return launch_pdl(k_bin, dim3((pd.n + threads - 1) / threads), dim3(threads), 0, s, dim, wide, g, ph.shell_h, tl, pd);
 }
 
 long long pack_block_bytes(int rec_double, int cap) {
@@ -154,15 +154,18 @@ long long pack_block_bytes(int rec_double, int cap) {
                       : block_elems<float>(cap) * (long long)sizeof(float);
 }
 
-cudaError_t launch_pack(int lattice, int rec_double, const Geom &g, const Tiles &tl, const Parts &pd,
-                        long long ntiles, cudaStream_t s) {
-    const dim3 blocks((unsigned)((g.nt[0] + kWarps - 1) / kWarps), (unsigned)g.nt[1], (unsigned)g.nt[2]);
-    if (lattice == 9) {
-        return rec_double ? launch_pdl(k_pack_tiles<D2Q9, double>, blocks, dim3(kThreads), 0, s, g, tl, pd, ntiles)
-                          : launch_pdl(k_pack_tiles<D2Q9, float>, blocks, dim3(kThreads), 0, s, g, tl, pd, ntiles);
-    }
-    return rec_double ? launch_pdl(k_pack_tiles<D3Q19, double>, blocks, dim3(kThreads), 0, s, g, tl, pd, ntiles)
-                      : launch_pdl(k_pack_tiles<D3Q19, float>, blocks, dim3(kThreads), 0, s, g, tl, pd, ntiles);
+template <class L, typename T>
+static cudaError_t launch_pack_t(const Geom &g, const Tiles &tl, const Parts &pd, long long ntiles, cudaStream_t s) {
+    // 8 tiles along x per block; y in the x grid too (its extent may exceed a y grid's)
+    const dim3 blocks((unsigned)((g.nt[0] + kWarps - 1) / kWarps) * (unsigned)g.nt[1], 1, (unsigned)g.nt[2]);
+    return launch_pdl(k_pack_tiles<L, T>, blocks, dim3(kThreads), 0, s, g, tl, pd, ntiles);
+}
+cudaError_t launch_pack(int lattice, int storage, const Geom &g, const Tiles &tl, const Parts &pd, long long ntiles,
+                        cudaStream_t s) {
+    const bool d2 = lattice == 9;
+    if (storage == ST_F64) return d2 ? launch_pack_t<D2Q9, double>(g, tl, pd, ntiles, s) : launch_pack_t<D3Q19, double>(g, tl, pd, ntiles, s);
+    if (!d2 && wide_tiles(3, storage == ST_F32 ? 4 : 2, g)) return launch_pack_t<D3Q19w, float>(g, tl, pd, ntiles, s);
+    return d2 ? launch_pack_t<D2Q9, float>(g, tl, pd, ntiles, s) : launch_pack_t<D3Q19, float>(g, tl, pd, ntiles, s);
 }
 
 cudaError_t launch_f_of_r(int dim, const double *R, double *Fr, int n, cudaStream_t s) {

@@ -73,10 +73,22 @@ __host__ inline void set_face_kind(Geom &g, const int a, const int hi, const int
     const int sh = 6 * a + 3 * hi;
     g.faces = (g.faces & ~(7 << sh)) | (kind << sh);
 }
-// Tile extent along axis ax: 32 x 8 x 1 cells for D2Q9, 32 x 4 x 2 for D3Q19 (one tile is
-// one thread block of the single-cell kernels).
-__host__ __device__ inline int tile_ext(const int dim, const int ax) {
-    return dim == 2 ? (ax == 0 ? 32 : (ax == 1 ? 8 : 1)) : (ax == 0 ? 32 : (ax == 1 ? 4 : 2));
+// Whether some face is open, an inlet or an outlet.
+__host__ __device__ inline bool open_faces(const Geom &g) {
+    bool any = false;
+    for (int a = 0; a < 3; ++a) any |= face_kind(g, a, 0) >= FACE_OPEN || face_kind(g, a, 1) >= FACE_OPEN;
+    return any;
+}
+// Whether a lattice is cut into the wide tiles (Tiled<> in lattice.cuh).
+__host__ __device__ inline int wide_tiles(const int dim, const size_t elem_bytes, const Geom &g) {
+    return elem_bytes == 4 && dim == 3 && !open_faces(g);
+}
+// Tile extent along axis ax: 32 x 8 x 1 cells for D2Q9, 32 x 4 x 2 for D3Q19; wide tiles 64 x 4 x 1
+// and 64 x 2 x 2. One tile is one thread block of the single-cell kernels.
+__host__ __device__ inline int tile_ext(const int dim, const int wide, const int ax) {
+    if (ax == 0) return wide ? 64 : 32;
+    if (ax == 1) return (dim == 2 ? 8 : 4) >> wide;
+    return dim == 2 ? 1 : 2;
 }
 
 // Physical parameters (FP64 on the host; kernels convert to their compute type).
@@ -97,15 +109,18 @@ struct Tiles {
     int *list;
     int cap;
     int *stats;          // [0] tiles that overflowed cap, [1] largest count, [2] length of
-                         // the overflow list, [3] [6] work counters of the collide-stream
-                         // kernel over the fluid and the particle tiles (zero between
-                         // launches), [4] tiles with candidates, [5] tiles without
+                         // the overflow list, [3] [6] work counters of the 16-bit kernels over
+                         // the fluid and the particle tiles (zero between launches), [4] tiles with candidates, [5] tiles without
+    int *work;           // work counters of the step's kernel (zero between launches): [0]
+                         // blocks that left, then kCounters of them, a cache line each
     void *blocks;        // per-tile packed candidate records (compute type), see psc_kernels.cuh
-    uint2 *order;        // [3 * ntiles] {tile id, ty | tz << 16}: tiles with candidates, then
-                         // (from ntiles on) tiles without, then (from 2 ntiles on) tiles with
-                         // more than cap; each list in rising id order within a block of 8
+    unsigned *order;     // [3 * ntiles] tile numbers: tiles with candidates, then (from ntiles
+                         // on) tiles without, then (from 2 ntiles on) tiles with more than
+                         // cap; each list in rising order within a block of 8
 };
 constexpr int kTileStats = 8;
+constexpr int kCounters = 32, kCounterStride = 32;
+constexpr int kWorkWords = (1 + kCounters) * kCounterStride;
 
 // Particle state on the device (FP64), and the force/torque accumulators (Eq. 14).
 struct Parts {
@@ -146,10 +161,10 @@ cudaError_t launch_gather(int storage, int lattice, const void *fin, double *f_o
 cudaError_t launch_set(int storage, int lattice, const double *f, void *fout,
                        const Geom &g, const Phys &ph, cudaStream_t s);
 // Bin particles into tile candidate lists and zero F, T.
-cudaError_t launch_bin(int dim, const Geom &g, const Phys &ph, const Tiles &tl,
+cudaError_t launch_bin(int dim, int wide, const Geom &g, const Phys &ph, const Tiles &tl,
                        const Parts &pd, cudaStream_t s);
-// Sort each tile's list and write its packed candidate records (rec_double: FP64 records).
-cudaError_t launch_pack(int lattice, int rec_double, const Geom &g, const Tiles &tl, const Parts &pd,
+// Sort each tile's list and write its packed candidate records (in the storage's compute type).
+cudaError_t launch_pack(int lattice, int storage, const Geom &g, const Tiles &tl, const Parts &pd,
                         long long ntiles, cudaStream_t s);
 // Bytes of one tile's packed block for the given candidate capacity.
 long long pack_block_bytes(int rec_double, int cap);

@@ -1,22 +1,22 @@
 // psc_kernels.cuh -- sm_103a kernels of one lattice-Boltzmann step with the modified
 // partially-saturated-cell (PSC) immersed moving boundary (Liu & Wu, arXiv 1901.09745).
 //
-// The lattice is cut into tiles (32 x 8 cells in 2D, 32 x 4 x 2 in 3D). After binning,
-// k_pack_tiles writes each tile's candidate particles as packed records and sorts the
-// tiles into three lists: tiles without candidates (k_fluid_pair: BGK + Guo + pull only),
-// tiles with at most 32 (k_collide_stream, psc_pair.cuh), tiles with more (the exact
-// chunked path of k_collide_overflow, psc_tile below). Per cell every path
+// The lattice is cut into tiles of 256 cells (tile_ext). After binning, k_pack_tiles writes each
+// tile's candidate particles as packed records and sorts the tiles into three lists: tiles
+// without candidates, tiles with at most 32 (both by k_step in psc_pair.cuh, 16-bit storage by
+// the kernels of psc_pair16.cuh), tiles with more (the exact chunked path of k_collide_overflow,
+// psc_tile below). Per cell every path
 //   1. pulls the Q post-collision populations of the previous step from the neighbours
 //      x - e_i (Eq. 1; periodic wrap; halfway bounce-back at walls, Eq. 6),
 //   2. forms rho and the force-shifted u (Eq. 5),
-//   3. walks the tile's candidate particles held in shared memory and computes each
-//      particle's solid fraction by the linear approximation (Eq. 15-18, Table 1),
+//   3. walks the tile's candidate particles and computes each particle's solid fraction by the
+//      linear approximation (Eq. 15-18, Table 1),
 //   4. forms eps_n, B_n (Eq. 9) and the per-particle weights B_{n,s} (Eq. 13),
 //   5. collides with BGK + Guo forcing + sum_s B_{n,s} Omega^s (Eq. 2-4, 10, 12) and
 //      stores the Q post-collision populations of its own cell,
 //   6. reduces each particle's momentum exchange B_{n,s} sum_i Omega^s_i e_i and its
-//      torque (Eq. 14) over the warp with shuffles, over the block in shared memory, and
-//      adds the block's total with one FP64 atomic per particle and component.
+//      torque (Eq. 14) over the warp with shuffles (16 bits and psc_tile: then over the block)
+//      and adds the total with one FP64 atomic per particle and component.
 //
 // Two algebraic identities keep the per-candidate work independent of Q (exact up to
 // rounding order, derived from Eq. 3 and Eq. 10):
@@ -48,6 +48,8 @@ template <typename T> struct PhysT {
     T F[3];         // body force
     T h;            // Table 1 shell half-width
     float2 sc;      // (scale, 1/scale) of the stored deviations
+    T none;         // 0, unknown to the compiler
+    T c12[2];       // 1 / 12 in the compute type and what that rounding left
     int inax;       // axis whose low face is an inlet (-1: none)
     T inua;         // inlet velocity along that axis
     T ineu[19];     // 6 w_i (e_i . u_in): f^eq_i - f^eq_{-i} of Eq. 3 at rho = 1
@@ -61,6 +63,9 @@ template <typename T> __host__ PhysT<T> make_phys(const Phys &ph, const int latt
     for (int a = 0; a < 3; ++a) k.F[a] = (T)ph.body_force[a];
     k.h = (T)ph.shell_h;
     k.sc = make_float2((float)ph.scale, (float)(1.0 / ph.scale));
+    k.none = (T)0;
+    k.c12[0] = (T)(1.0 / 12.0);
+    k.c12[1] = (T)(1.0 / 12.0 - (double)k.c12[0]);
     const double *u = ph.inflow;
     k.inax = ph.inflow_axis;
     k.inua = (T)(ph.inflow_axis >= 0 ? u[ph.inflow_axis] : 0.0);   // the inlet is a low face
@@ -188,10 +193,14 @@ pull_one(const S *__restrict__ fin, const Geom &g, int x, int y, int z, long lon
 // as 0, `from_inlet` or `from_outlet` set) and is filled in by inflow_nebb or outlet_nebb
 // once all are pulled. A wall takes precedence over the inlet and outlet faces, these over
 // open faces.
-template <class L, typename S>
+template <class L, typename S, bool RAW = false>
 __device__ __forceinline__ typename Store<S>::T
 pull_one_faces(const S *__restrict__ fin, const Geom &g, int x, int y, int z, long long cell, int i,
                float2 sc, bool &from_inlet, bool &from_outlet) {
+    auto ld = [&](long long k) {
+        const long long c = PSC_IDX(k, L::Q * g.ncell, CHK_POP);
+        return RAW ? Store<S>::ldr(fin, c) : Store<S>::ld(fin, c, sc);
+    };
     int s[3] = {x - L::ex(i), y - L::ey(i), z - L::ez(i)};
     bool bounce = false, inflow = false, outflow = false;
 #pragma unroll
@@ -205,17 +214,17 @@ pull_one_faces(const S *__restrict__ fin, const Geom &g, int x, int y, int z, lo
             else outflow = true;
         }
     }
-    if (bounce) return Store<S>::ld(fin, PSC_IDX((long long)opp<L>(i) * g.ncell + cell, L::Q * g.ncell, CHK_POP), sc);
+    if (bounce) return ld((long long)opp<L>(i) * g.ncell + cell);
     from_inlet = inflow;
     from_outlet = outflow && !inflow;
     if (inflow || outflow) return (typename Store<S>::T)0;
     long long src = (long long)s[0] + (long long)g.n[0] * ((long long)s[1] + (long long)g.n[1] * s[2]);
-    return Store<S>::ld(fin, PSC_IDX((long long)i * g.ncell + src, L::Q * g.ncell, CHK_POP), sc);
+    return ld((long long)i * g.ncell + src);
 }
 
 // All Q populations of cell (x, y, z) after streaming, one pull_one per direction, the
 // unknown ones at an inlet filled in.
-template <class L, typename S>
+template <class L, typename S, bool RAW = false>
 __device__ __forceinline__ void pull_all(const S *__restrict__ fin, const Geom &g, int x, int y, int z,
                                          long long cell, const PhysT<typename Store<S>::T> &ph,
                                          typename Store<S>::T *df) {
@@ -223,12 +232,12 @@ __device__ __forceinline__ void pull_all(const S *__restrict__ fin, const Geom &
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
         bool in = false, out = false;
-        df[i] = pull_one_faces<L, S>(fin, g, x, y, z, cell, i, ph.sc, in, out);
+        df[i] = pull_one_faces<L, S, RAW>(fin, g, x, y, z, cell, i, ph.sc, in, out);
         if (in) fill |= 1u << i;
         if (out) fillo |= 1u << i;
     }
-    if (fill) inflow_nebb<L, false>(df, ph, ph.sc, fill);
-    if (fillo) outlet_nebb<L, false>(df, ph, ph.sc, fillo);
+    if (fill) inflow_nebb<L, RAW>(df, ph, ph.sc, fill);
+    if (fillo) outlet_nebb<L, RAW>(df, ph, ph.sc, fillo);
 }
 
 // Warp sum of NV values per lane (NV a power of two <= 32) in NV - 1 + 5 - log2(NV) shuffles
@@ -376,7 +385,6 @@ __device__ __forceinline__ void pull_q(const S *__restrict__ fin, const Geom &g,
 // loads, so the candidate table costs no extra latency on the critical path.
 constexpr int RW = 12;
 enum { R_PX = 0, R_PY, R_PZ, R_R, R_FR, R_UX, R_UY, R_UZ, R_OX, R_OY, R_OZ, R_ID };
-constexpr int kPre = 16;
 
 template <typename T> __host__ __device__ constexpr int head_elems() { return 16 / (int)sizeof(T); }
 template <typename T> __host__ __device__ inline long long block_elems(int cap) {
@@ -404,7 +412,7 @@ __device__ __forceinline__ void write_record(T *rec, const Geom &g, const Parts 
         T rel = (T)0;
         if (a < L::D) {
             // minimum image with respect to the tile centre, one exact FP64 subtraction
-            rel = (T)record_rel(pd.X[3 * id + a], org[a], ext[a], g.n[a], g.inv_n[a], g.periodic[a]);
+            rel = (T)(record_rel(pd.X[3 * id + a], org[a], ext[a], g.n[a], g.inv_n[a], g.periodic[a]) - (a == 0 ? L::REC_X : 0));
         }
         rec[R_PX + a] = rel;
     }
@@ -419,6 +427,11 @@ __device__ __forceinline__ void write_record(T *rec, const Geom &g, const Parts 
         rec[R_UX] = (T)pd.U[3 * id + 0]; rec[R_UY] = (T)pd.U[3 * id + 1]; rec[R_UZ] = (T)pd.U[3 * id + 2];
         rec[R_OX] = (T)pd.Om[3 * id + 0]; rec[R_OY] = (T)pd.Om[3 * id + 1]; rec[R_OZ] = (T)pd.Om[3 * id + 2];
     }
+    // f(r) > 0: a negative one marks a particle that moves or spins
+    bool moves = false;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) moves |= (rec[R_UX + a] != (T)0) || (rec[R_OX + a] != (T)0);
+    if (moves) rec[R_FR] = -rec[R_FR];
     rec[R_ID] = id_bits<T>(id);
 }
 
@@ -432,12 +445,12 @@ template <class L, typename T>
 __global__ void k_pack_tiles(Geom g, Tiles tl, Parts pd, long long ntiles) {
     __shared__ int s_id[kWarps][64];
     __shared__ int s_cnt[kWarps];
-    __shared__ uint2 s_ent[kWarps];
     pdl_wait();       // the binning kernel's counts and lists
     pdl_launch();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // grid (nt0 / 8, nt1, nt2): the block's 8 warps take 8 tiles along x, no division
-    const int tx = (int)blockIdx.x * kWarps + warp, ty = (int)blockIdx.y, tz = (int)blockIdx.z;
+    // grid (nt0 / 8 * nt1, 1, nt2): the block's 8 warps take 8 tiles along x
+    const unsigned nbx = (unsigned)(g.nt[0] + kWarps - 1) / kWarps, by = blockIdx.x / nbx;
+    const int tx = (int)(blockIdx.x - by * nbx) * kWarps + warp, ty = (int)by, tz = (int)blockIdx.z;
     const long long tile = tx + (long long)g.nt[0] * (ty + (long long)g.nt[1] * tz);
     const bool valid = tx < g.nt[0];
     const int cnt = valid ? tl.count[tile] : -1;
@@ -448,7 +461,6 @@ __global__ void k_pack_tiles(Geom g, Tiles tl, Parts pd, long long ntiles) {
         if (lane == 0) blk[0] = (T)cnt;
         for (int k = lane; k < m; k += 32) s_id[warp][k] = tl.list[tile * tl.cap + k];
         __syncwarp();
-        if (lane == 0) s_ent[warp] = make_uint2((unsigned)tile, (unsigned)ty | ((unsigned)tz << 16));
         for (int k = lane; k < m; k += 32) {
             const int id = (int)PSC_IDX(s_id[warp][k], pd.n, CHK_PART);
             int rank = 0;
@@ -469,7 +481,7 @@ __global__ void k_pack_tiles(Geom g, Tiles tl, Parts pd, long long ntiles) {
         int bo = no ? atomicAdd(&tl.stats[2], no) : 0;
         for (int w = 0; w < kWarps; ++w) {
             if (s_cnt[w] < 0) continue;
-            const uint2 ent = s_ent[w];
+            const unsigned ent = (unsigned)(tile + w);      // thread 0's warp is the first
             if (s_cnt[w] > 0) tl.order[bp++] = ent;
             else tl.order[ntiles + bf++] = ent;
             if (s_cnt[w] > lim) tl.order[2 * ntiles + bo++] = ent;
@@ -491,32 +503,6 @@ template <> __device__ __forceinline__ Vec4<double> ld4<double>(const double *p)
     return {a.x, a.y, b.x, b.y};
 }
 
-// Solid fraction of the candidate in record `rec` at the cell with tile-relative centre
-// (cx, cy, cz): Table 1 Steps 2-4 with the inside/outside branches as stated in Sec. 2.4
-// (distance <= r - h -> 1, >= r + h -> 0), else clamp(f(r) - D, 0, 1) with D = distance - r
-// (Eq. 15). Returns 0 outside; on return (dx, dy, dz) is the arm x_n - X_p.
-template <class L, typename T>
-__device__ __forceinline__ T cand_eps(const T *rec, const Geom &g, T cx, T cy, T cz, T h, T &dx, T &dy,
-                                      T &dz) {
-    const Vec4<T> pr = ld4<T>(rec);                      // px, py, pz, r
-    dx = cx - pr.x;
-    dy = cy - pr.y;
-    dz = (L::D == 3) ? cz - pr.z : (T)0;
-    if (g.wrap_img[0]) dx -= (T)g.n[0] * rint_t(dx / (T)g.n[0]);
-    if (g.wrap_img[1]) dy -= (T)g.n[1] * rint_t(dy / (T)g.n[1]);
-    if (L::D == 3 && g.wrap_img[2]) dz -= (T)g.n[2] * rint_t(dz / (T)g.n[2]);
-    const T d2 = dx * dx + dy * dy + dz * dz;
-    const T r = pr.w;
-    const T rh = r + h;
-    if (!(d2 < rh * rh)) return (T)0;
-    const T dist = sqrt_t(d2);
-    if (dist <= r - h) return (T)1;
-    T e = rec[R_FR] - (dist - r);
-    e = e < (T)0 ? (T)0 : e;
-    e = e > (T)1 ? (T)1 : e;
-    return e;
-}
-
 // Arm x_n - X_p from the cell (cx, cy, cz) to the candidate at (px, py, pz), all relative
 // to the tile origin, with the per-cell minimum image on short periodic axes.
 template <class L, typename T>
@@ -534,6 +520,7 @@ __device__ __forceinline__ void cand_arm(const Geom &g, T cx, T cy, T cz, T px, 
 // distance <= r - h -> 1, >= r + h -> 0, else clamp(f(r) - D, 0, 1) with D = distance - r.
 template <typename T>
 __device__ __forceinline__ T shell_eps(T d2, T r, T fr, T h) {
+    fr = fabs(fr);      // a record marks moving particles by the sign
     const T rh = r + h;
     if (!(d2 < rh * rh)) return (T)0;
     const T ri = r - h;
@@ -559,10 +546,6 @@ __device__ __forceinline__ bool row_hits(const Geom &g, T px, T py, T pz, T R, T
     return (px - hw <= xmax + (T)1) && (px + hw >= (T)-1);
 }
 
-template <class L, typename T> constexpr int psc_min_blocks() {
-    return sizeof(T) == 8 ? 1 : (L::Q == 9 ? 4 : 3);
-}
-
 // Tiles with candidate particles. The tile's records are staged in shared memory while the
 // population loads are in flight. Each warp is one row of the tile: it culls the candidates
 // that cannot reach its row (one lane per candidate, ballot), then every lane evaluates the
@@ -571,7 +554,7 @@ template <class L, typename T> constexpr int psc_min_blocks() {
 // shuffles; partial sums meet in shared memory and are added in a fixed order, one FP64
 // atomic per particle and component per tile. Tiles with more candidates than the block
 // holds take the same path chunk by chunk over all particles (exact, slow, rare).
-template <class L, typename S, int PSC, bool FACES = false>
+template <class L, typename S, int PSC, bool FACES = false, bool FLUID = false>
 __device__ __forceinline__ void psc_tile(const unsigned tile, const S *__restrict__ fin, S *__restrict__ fout,
                                          const Geom &g, const PhysT<typename Store<S>::T> &ph, const Tiles &tl,
                                          const Parts &pd, int *flags, typename Store<S>::T *srec,
@@ -583,16 +566,15 @@ __device__ __forceinline__ void psc_tile(const unsigned tile, const S *__restric
     const int cap = tl.cap;
     T *part = srec + (size_t)cap * RW;                     // [kWarps][cap][NC] warp partials
 
-    // (without particles the tile lists may not exist: only the faces kernel gets here then)
-    const int cnt = (FACES && pd.n == 0) ? 0 : tl.count[tile];
-    if (cnt == 0 && !FACES) return;                        // plain-fluid tile: k_fluid_pair does it
+    // (FLUID: a tile without candidates)
+    const int cnt = FLUID ? 0 : tl.count[tile];
     const unsigned txy = tile / (unsigned)g.nt[0];          // 32-bit: tiles < 2^31 (host check)
     const int tx = (int)(tile - txy * (unsigned)g.nt[0]);
     const int ty = (int)(txy % (unsigned)g.nt[1]);
     const int tz = (int)(txy / (unsigned)g.nt[1]);
     const bool ovf = cnt > cap;
     const int nchunk = ovf ? (pd.n + cap - 1) / cap : 1;
-    const T *recs = (FACES && cnt == 0) ? nullptr
+    const T *recs = FLUID ? nullptr
                   : reinterpret_cast<const T *>(tl.blocks) + (size_t)tile * block_elems<T>(cap) + head_elems<T>();
 
     const int tid = threadIdx.x + L::TX * (threadIdx.y + L::TY * threadIdx.z);
@@ -659,7 +641,7 @@ __device__ __forceinline__ void psc_tile(const unsigned tile, const S *__restric
     }
 
     // ---- 3. candidates reaching this row: solid fractions and u_s moments of the cell
-    const T cx = (T)threadIdx.x, cy = (T)threadIdx.y, cz = (T)threadIdx.z;
+    const T cx = (T)((int)threadIdx.x - L::REC_X), cy = (T)threadIdx.y, cz = (T)threadIdx.z;
     const T xmax = (T)(min(L::TX, g.n[0] - x0) - 1);
     T seps = 0, mx = 0, my = 0, mz = 0, Mxx = 0, Myy = 0, Mzz = 0, Mxy = 0, Mxz = 0, Myz = 0;
     unsigned long long wmask = 0ull;     // relevant candidates of this row (normal tiles)
@@ -678,7 +660,7 @@ __device__ __forceinline__ void psc_tile(const unsigned tile, const S *__restric
             bool rel = false;
             if (k < nk) {
                 const Vec4<T> a = ld4<T>(srec + k * RW);
-                rel = row_hits<L, T>(g, a.x, a.y, a.z, a.w + ph.h, cy, cz, xmax);
+                rel = row_hits<L, T>(g, a.x + (T)L::REC_X, a.y, a.z, a.w + ph.h, cy, cz, xmax);
             }
             unsigned bal = __ballot_sync(kFull, rel);
             if (!ovf) wmask |= (unsigned long long)bal << kb;
@@ -797,7 +779,7 @@ __device__ __forceinline__ void psc_tile(const unsigned tile, const S *__restric
                     rel = false;
                     if (k < nk) {
                         write_record<L, T>(ovr, g, pd, ch * cap + k, x0, y0, z0);
-                        rel = row_hits<L, T>(g, ovr[R_PX], ovr[R_PY], ovr[R_PZ], ovr[R_R] + ph.h, cy, cz, xmax);
+                        rel = row_hits<L, T>(g, ovr[R_PX] + (T)L::REC_X, ovr[R_PY], ovr[R_PZ], ovr[R_R] + ph.h, cy, cz, xmax);
                     }
                 }
                 unsigned bal = __ballot_sync(kFull, rel);
@@ -892,6 +874,7 @@ __device__ __forceinline__ void psc_tile(const unsigned tile, const S *__restric
 }
 
 #include "psc_pair.cuh"
+#include "psc_pair16.cuh"
 
 // Tiles with more candidates than the block holds (rare): the exact chunked path over all
 // particles, one block per tile of the overflow list. With no such tile every block returns
@@ -905,31 +888,34 @@ k_collide_overflow(const S *__restrict__ fin, S *__restrict__ fout, Geom g, Phys
     __shared__ unsigned long long s_mask[kWarps];
     const long long ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
     const int novf = tl.stats[2];
-    // the collide-stream kernel before this one has finished: clear its work counters
+    // the 16-bit kernel before this one has finished: clear its work counters
     if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) {
         tl.stats[3] = 0;
         tl.stats[6] = 0;
     }
     for (int it = blockIdx.x; it < novf; it += gridDim.x) {
-        psc_tile<L, S, PSC>(tl.order[2 * ntiles + it].x, fin, fout, g, ph, tl, pd, flags,
-                            reinterpret_cast<T *>(smem), s_mask);
+        psc_tile<L, S, PSC>(tl.order[2 * ntiles + it], fin, fout, g, ph, tl, pd, flags, reinterpret_cast<T *>(smem), s_mask);
         __syncthreads();
     }
 }
 
-// Contexts with an open, inlet or outlet face: every tile, with or without candidates, by
-// the single-cell path whose pull classifies each face (persistent blocks over the tiles).
-template <class L, typename S, int PSC>
-__global__ void __launch_bounds__(kThreads, 1)
+// Contexts with an open, inlet or outlet face, by the single-cell path whose pull classifies each
+// face (blocks striding over the tiles): SOLID the list of tiles with candidates, else those
+// without (every tile when there are no particles). Apart, the tiles without need a third of
+// the registers, so three blocks instead of one share an SM: a box of 120 x 60 x 60 with one
+// sphere takes 65 us a step where one kernel for both took 104.
+template <class L, typename S, int PSC, bool SOLID>
+__global__ void __launch_bounds__(kThreads, SOLID ? 1 : (sizeof(S) == 8 ? 2 : 3))
 k_collide_faces(const S *__restrict__ fin, S *__restrict__ fout, Geom g, PhysT<typename Store<S>::T> ph,
                 Tiles tl, Parts pd, int *flags) {
     using T = typename Store<S>::T;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long s_mask[kWarps];
-    const long long ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
-    for (long long it = blockIdx.x; it < ntiles; it += gridDim.x) {
-        psc_tile<L, S, PSC, true>((unsigned)it, fin, fout, g, ph, tl, pd, flags,
-                                  reinterpret_cast<T *>(smem), s_mask);
+    const unsigned ntiles = (unsigned)g.nt[0] * (unsigned)g.nt[1] * (unsigned)g.nt[2];
+    const unsigned n = SOLID ? (unsigned)tl.stats[4] : (pd.n > 0 ? (unsigned)tl.stats[5] : ntiles);
+    for (unsigned it = blockIdx.x; it < n; it += gridDim.x) {
+        const unsigned tile = SOLID ? tl.order[it] : (pd.n > 0 ? tl.order[ntiles + it] : it);
+        psc_tile<L, S, PSC, true, !SOLID>(tile, fin, fout, g, ph, tl, pd, flags, reinterpret_cast<T *>(smem), s_mask);
         __syncthreads();
     }
 }
@@ -1026,9 +1012,11 @@ k_macro(const S *__restrict__ fin, Geom g, PhysT<typename Store<S>::T> ph, doubl
     using T = typename Store<S>::T;
     __shared__ double s_u[kWarps][3 * 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int x0 = blockIdx.x * L::TX, y0 = blockIdx.y * L::TY, z0 = blockIdx.z * L::TZ;
-    const int x = x0 + lane, y = y0 + warp % L::TY, z = z0 + warp / L::TY;
-    if (y >= g.n[1] || z >= g.n[2]) return;       // the whole warp
+    // grid (nt0 * nt1, 1, nt2); a warp takes 32 cells of a row
+    const int ty = (int)(blockIdx.x / (unsigned)g.nt[0]), row_of = warp / (L::TX / 32);
+    const int x0 = (int)(blockIdx.x - (unsigned)ty * (unsigned)g.nt[0]) * L::TX + 32 * (warp % (L::TX / 32));
+    const int x = x0 + lane, y = ty * L::TY + row_of % L::TY, z = (int)blockIdx.z * L::TZ + row_of / L::TY;
+    if (x0 >= g.n[0] || y >= g.n[1] || z >= g.n[2]) return;       // the whole warp
     const bool in = x < g.n[0];
     const long long row = (long long)g.n[0] * (y + (long long)g.n[1] * z);
     const long long cell = row + x;
@@ -1036,8 +1024,8 @@ k_macro(const S *__restrict__ fin, Geom g, PhysT<typename Store<S>::T> ph, doubl
     if (FACES) {
         if (in) pull_all<L, S>(fin, g, x, y, z, cell, ph, df);
     } else {
-        const bool interior = x0 >= 1 && x0 + L::TX < g.n[0] && y0 >= 1 && y0 + L::TY < g.n[1] &&
-                              (L::D == 2 || (z0 >= 1 && z0 + L::TZ < g.n[2]));
+        const bool interior = x0 >= 1 && x0 + 32 < g.n[0] && y >= 1 && y + 1 < g.n[1] &&
+                              (L::D == 2 || (z >= 1 && z + 1 < g.n[2]));
         pull_q<L, S>(fin, g, x, y, z, cell, interior, in, ph.sc, df);
     }
     const int count = min(32, g.n[0] - x0);
@@ -1122,23 +1110,95 @@ inline cudaError_t persistent_blocks(K kern, size_t smem, long long work, unsign
                                      int *per_sm = nullptr) {
     static thread_local const void *c_kern = nullptr;
     static thread_local size_t c_smem = (size_t)-1;
-    static thread_local int c_per = 0;
+    static thread_local int c_per = 0, c_threads = 0;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (c_smem != smem || c_kern != (const void *)kern) {
+    if (c_smem != smem || c_kern != (const void *)kern || c_threads != threads) {
         int per = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, threads, smem);
         if (e != cudaSuccess) return e;
         c_per = per > 0 ? per : 1;
         c_smem = smem;
         c_kern = (const void *)kern;
+        c_threads = threads;
     }
     const long long b = (long long)sms * c_per;
     blocks = (unsigned)(b < work ? b : (work > 0 ? work : 1));
     if (per_sm) *per_sm = c_per;
     return cudaSuccess;
+}
+
+// The overflow-tile kernel (tiles with more candidates than the step's kernel keeps), which
+// also clears that kernel's work counters for the next launch.
+template <class L, typename S, int PSC>
+cudaError_t launch_overflow(const void *fin, void *fout, const Geom &g, const PhysT<typename Store<S>::T> &pt,
+                            const Tiles &tl, const Parts &pd, int *flags, cudaStream_t s) {
+    using T = typename Store<S>::T;
+    constexpr int NC = (L::D == 2) ? 3 : 6;
+    const size_t osmem = cs_smem_bytes<T>(tl.cap, NC);
+    auto okern = k_collide_overflow<L, S, PSC>;
+    if (osmem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(okern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osmem);
+        if (e != cudaSuccess) return e;
+    }
+    okern<<<32, dim3(L::TX, L::TY, L::TZ), osmem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
+    return cudaGetLastError();
+}
+
+// Fluid-tile blocks per SM when they follow the particle tiles beside the caller's next
+// kernels (a deferred join).
+constexpr int kDeferF = 2;
+
+// One launch of the step's kernel over the tiles of kind `which` (blocks_per_sm > 0 limits it).
+template <class L, typename S, int PSC, bool SOLID, bool VEC>
+cudaError_t launch_step_t(const void *fin, void *fout, const Geom &g, const PhysT<typename Store<S>::T> &pt,
+                          const Tiles &tl, const Parts &pd, int *flags, int which, int blocks_per_sm, cudaStream_t s) {
+    auto kern = k_step<L, S, PSC, SOLID, VEC>;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const long long ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
+    // a whole tile per item where every warp of a full chip gets many (256^3: 431 us against 442),
+    // else a unit (2048^2 FP16 64 against 69, 777 x 453 19 against 28); few items go to blocks of
+    // one warp, spread over the SMs
+    const int shift = ntiles >= 16LL * 16 * sms ? 0 : 2;
+    const long long items = ntiles << shift;
+    const int threads = items <= 8LL * sms ? 32 : kPThreads;
+    unsigned nb = 0;
+    e = persistent_blocks(kern, 0, (items + threads / 32 - 1) / (threads / 32), nb, threads);
+    if (e != cudaSuccess) return e;
+    if (blocks_per_sm > 0 && nb > (unsigned)(blocks_per_sm * sms)) nb = (unsigned)(blocks_per_sm * sms);
+    kern<<<nb, threads, 0, s>>>(Dirs<L, S>(fin, fout, g), g, pt, tl, pd, flags, tl.work, which, shift);
+    return cudaGetLastError();
+}
+
+// One collide-stream step. Without particles: the fluid kernel over every tile. With
+// particles: one kernel over the tiles with candidates and then those without, and the
+// overflow kernel. In a coupled step (ov->defer; 2D, FP32 and 16-bit storage) the tiles with
+// candidates and the overflow tiles first, then those without on the second stream, a few
+// blocks per SM, beside the caller's next kernels.
+template <class L, typename S, int PSC, bool VEC>
+cudaError_t launch_collide_stream_t(const void *fin, void *fout, const Geom &g, const Phys &ph,
+                                    const Tiles &tl, const Parts &pd, int *flags, cudaStream_t s,
+                                    Overlap *ov) {
+    using T = typename Store<S>::T;
+    const PhysT<T> pt = make_phys<T>(ph, L::Q);
+    if (pd.n == 0) return launch_step_t<L, S, 0, false, VEC>(fin, fout, g, pt, tl, pd, flags, kAllTiles, 0, s);
+    const bool defer = ov && ov->aux && ov->defer && L::D == 2 && sizeof(T) == 4;
+    cudaError_t e = launch_step_t<L, S, PSC, true, VEC>(fin, fout, g, pt, tl, pd, flags,
+                                                              defer ? kParticleTiles : kBothLists, 0, s);
+    if (e == cudaSuccess) e = launch_overflow<L, S, PSC>(fin, fout, g, pt, tl, pd, flags, s);
+    if (e != cudaSuccess || !defer) return e;
+    e = cudaEventRecord(ov->fork, s);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ov->aux, ov->fork, 0);
+    if (e == cudaSuccess)
+        e = launch_step_t<L, S, 0, false, VEC>(fin, fout, g, pt, tl, pd, flags, kFluidTiles, kDeferF, ov->aux);
+    if (e == cudaSuccess) e = cudaEventRecord(ov->join, ov->aux);
+    if (e == cudaSuccess) ov->deferred = 1;
+    return e;
 }
 
 // Registers a block of `threads` holds (allocated per warp in units of 8 per thread).
@@ -1150,72 +1210,34 @@ inline cudaError_t block_registers(K kern, int threads, int &regs) {
     return e;
 }
 
-// One collide-stream step. Without particles: the fluid kernel over every tile. With
-// The overflow-tile kernel (tiles with more candidates than the pair kernels keep), which also
-// clears the particle-tile kernel's work counters for the next launch.
-template <class L, typename S, int PSC>
-cudaError_t launch_overflow(const void *fin, void *fout, const Geom &g, const PhysT<typename Store<S>::T> &pt,
-                            const Tiles &tl, const Parts &pd, int *flags, size_t osmem, dim3 block, cudaStream_t s) {
-    auto okern = k_collide_overflow<L, S, PSC>;
-    if (osmem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(okern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osmem);
-        if (e != cudaSuccess) return e;
-    }
-    okern<<<32, block, osmem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
-    return cudaGetLastError();
-}
-
-// Fluid-tile blocks per SM when they follow the particle tiles beside the caller's next
-// kernels (a deferred join). On the 2048^2 channel with 5000 discs and its DEM call the
-// coupled step took 167.8 / 140.8 / 142.0 / 146.0 / 147.2 / 159.4 us with 1 / 2 / 3 / 4 / 5
-// / 6 blocks per SM (156 us as two calls): fewer leave the fluid tiles unfinished when the
-// DEM call ends, more slow the latency-bound DEM kernels down.
-constexpr int kDeferF = 2;
-
-// particles in 2D (FP32 and 16-bit storage): the particle-tile kernel (4 blocks per SM) and
+// 16-bit storage. Without particles: the fluid kernel over every tile. With particles in 2D: the particle-tile kernel (4 blocks per SM) and
 // the fluid-tile kernel (3 blocks per SM) side by side on two streams, which together fill
 // each SM's register file, so the issue-bound particle tiles and the DRAM-bound fluid tiles
 // share every SM for the whole step; without a second stream, one after the other. In 3D
-// (and FP64) the particle-tile kernel holds all the registers an SM has, and takes the
+// the particle-tile kernel holds all the registers an SM has, and takes the
 // fluid tiles itself once its own are done. Then the overflow kernel.
 template <class L, typename S, int PSC>
-cudaError_t launch_collide_stream_t(const void *fin, void *fout, const Geom &g, const Phys &ph,
+cudaError_t launch_collide_stream16(const void *fin, void *fout, const Geom &g, const Phys &ph,
                                     const Tiles &tl, const Parts &pd, int *flags, cudaStream_t s,
                                     Overlap *ov) {
     using T = typename Store<S>::T;
-    constexpr int NC = (L::D == 2) ? 3 : 6;
-    constexpr bool kSteal = (L::D == 3) || sizeof(T) == 8;
+    constexpr bool kSteal = L::D == 3;
     // blocks per SM side by side (2D): 4 x 128 threads x 80 registers + 3 x 128 x 64 = 64 K
     constexpr int kSideP = 4, kSideF = 3;
-    const size_t smem = pair_smem_bytes<L, T>();
-    const size_t osmem = cs_smem_bytes<T>(tl.cap, NC);
-    auto kern = k_collide_stream<L, S, PSC, kSteal>;
+    const size_t smem = h16::pair_smem_bytes<L, T>();
+    auto kern = h16::k_collide_stream<L, S, PSC, kSteal>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     const long long ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
-    dim3 block(L::TX, L::TY, L::TZ);
     const PhysT<T> pt = make_phys<T>(ph, L::Q);
-    bool faces = false;
-    for (int a = 0; a < 3; ++a) faces |= face_kind(g, a, 0) >= FACE_OPEN || face_kind(g, a, 1) >= FACE_OPEN;
-    if (faces) {
-        auto fk = k_collide_faces<L, S, PSC>;
-        if (osmem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(fk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osmem);
-            if (e != cudaSuccess) return e;
-        }
-        unsigned nbf = 0;
-        cudaError_t e = persistent_blocks(fk, osmem, ntiles, nbf, kThreads);
-        if (e != cudaSuccess) return e;
-        fk<<<nbf, block, osmem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
-        return cudaGetLastError();
-    }
+    const Dirs<L, S> f(fin, fout, g);
     const bool hasF = ph.body_force[0] != 0.0 || ph.body_force[1] != 0.0 || ph.body_force[2] != 0.0;
-    auto fkern = hasF ? k_fluid_pair<L, S, true> : k_fluid_pair<L, S, false>;
+    auto fkern = hasF ? h16::k_fluid_pair<L, S, true> : h16::k_fluid_pair<L, S, false>;
     const dim3 pblock(32, kPWarps);
     if (pd.n == 0) {
-        fkern<<<dim3(g.nt[0], g.nt[1], g.nt[2]), pblock, 0, s>>>((const S *)fin, (S *)fout, g, pt, tl, 0, flags);
+        fkern<<<dim3(g.nt[0], g.nt[1], g.nt[2]), pblock, 0, s>>>(f, g, pt, tl, 0, flags);
         return cudaGetLastError();
     }
     cudaError_t e;
@@ -1236,12 +1258,12 @@ cudaError_t launch_collide_stream_t(const void *fin, void *fout, const Geom &g, 
     if (side && ov->defer) {
         e = persistent_blocks(kern, smem, ntiles, nb, kPThreads);
         if (e != cudaSuccess) return e;
-        kern<<<nb, pblock, smem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
-        e = launch_overflow<L, S, PSC>(fin, fout, g, pt, tl, pd, flags, osmem, block, s);
+        kern<<<nb, pblock, smem, s>>>(f, g, pt, tl, pd, flags);
+        e = launch_overflow<L, S, PSC>(fin, fout, g, pt, tl, pd, flags, s);
         if (e == cudaSuccess) e = cudaEventRecord(ov->fork, s);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ov->aux, ov->fork, 0);
         if (e != cudaSuccess) return e;
-        fkern<<<nsm * kDeferF, pblock, 0, ov->aux>>>((const S *)fin, (S *)fout, g, pt, tl, pd.n, flags);
+        fkern<<<nsm * kDeferF, pblock, 0, ov->aux>>>(f, g, pt, tl, pd.n, flags);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaEventRecord(ov->join, ov->aux);
         if (e == cudaSuccess) ov->deferred = 1;
@@ -1251,8 +1273,8 @@ cudaError_t launch_collide_stream_t(const void *fin, void *fout, const Geom &g, 
         e = cudaEventRecord(ov->fork, s);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ov->aux, ov->fork, 0);
         if (e != cudaSuccess) return e;
-        kern<<<nsm * kSideP, pblock, smem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
-        fkern<<<nsm * kSideF, pblock, 0, ov->aux>>>((const S *)fin, (S *)fout, g, pt, tl, pd.n, flags);
+        kern<<<nsm * kSideP, pblock, smem, s>>>(f, g, pt, tl, pd, flags);
+        fkern<<<nsm * kSideF, pblock, 0, ov->aux>>>(f, g, pt, tl, pd.n, flags);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaEventRecord(ov->join, ov->aux);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s, ov->join, 0);
@@ -1261,15 +1283,54 @@ cudaError_t launch_collide_stream_t(const void *fin, void *fout, const Geom &g, 
         if (!kSteal) {
             e = persistent_blocks(fkern, 0, ntiles, nb, kPThreads);
             if (e != cudaSuccess) return e;
-            fkern<<<nb, pblock, 0, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd.n, flags);
+            fkern<<<nb, pblock, 0, s>>>(f, g, pt, tl, pd.n, flags);
         }
         e = persistent_blocks(kern, smem, ntiles, nb, kPThreads);
         if (e != cudaSuccess) return e;
-        kern<<<nb, pblock, smem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
+        kern<<<nb, pblock, smem, s>>>(f, g, pt, tl, pd, flags);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    return launch_overflow<L, S, PSC>(fin, fout, g, pt, tl, pd, flags, osmem, block, s);
+    return launch_overflow<L, S, PSC>(fin, fout, g, pt, tl, pd, flags, s);
+}
+
+template <class L, typename S, int PSC>
+cudaError_t launch_faces_t(const void *fin, void *fout, const Geom &g, const Phys &ph, const Tiles &tl, const Parts &pd,
+                           int *flags, cudaStream_t s) {
+    using T = typename Store<S>::T;
+    const PhysT<T> pt = make_phys<T>(ph, L::Q);
+    const dim3 block(L::TX, L::TY, L::TZ);
+    const long long ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
+    unsigned nb = 0;
+    if (pd.n > 0) {
+        auto kern = k_collide_faces<L, S, PSC, true>;
+        const size_t smem = cs_smem_bytes<T>(tl.cap, L::D == 2 ? 3 : 6);
+        cudaError_t e = cudaSuccess;
+        if (smem > 48 * 1024) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess) e = persistent_blocks(kern, smem, ntiles, nb, kThreads);
+        if (e != cudaSuccess) return e;
+        kern<<<nb, block, smem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
+    }
+    auto kern = k_collide_faces<L, S, PSC, false>;
+    cudaError_t e = persistent_blocks(kern, 0, ntiles, nb, kThreads);
+    if (e != cudaSuccess) return e;
+    kern<<<nb, block, 0, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
+    return cudaGetLastError();
+}
+
+template <class L, typename S, int PSC>
+cudaError_t launch_collide_stream_l(const void *fin, void *fout, const Geom &g, const Phys &ph, const Tiles &tl,
+                                    const Parts &pd, int *flags, cudaStream_t s, Overlap *ov) {
+    if (open_faces(g)) return launch_faces_t<L, S, PSC>(fin, fout, g, ph, tl, pd, flags, s);
+    if constexpr (sizeof(S) == 2) {
+        return launch_collide_stream16<L, S, PSC>(fin, fout, g, ph, tl, pd, flags, s, ov);
+    } else {
+        using W = Tiled<L, S>;
+        // pairs in one access: every row of every direction starts on a pair boundary
+        const bool vec = g.n[0] % 2 == 0 && ((uintptr_t)fin | (uintptr_t)fout) % (2 * sizeof(S)) == 0;
+        return vec ? launch_collide_stream_t<W, S, PSC, true>(fin, fout, g, ph, tl, pd, flags, s, ov)
+                   : launch_collide_stream_t<W, S, PSC, false>(fin, fout, g, ph, tl, pd, flags, s, ov);
+    }
 }
 
 template <typename S>
@@ -1277,20 +1338,18 @@ cudaError_t launch_collide_stream_storage(int lattice, const void *fin, void *fo
                                           const Phys &ph, const Tiles &tl, const Parts &pd,
                                           int *flags, cudaStream_t s, Overlap *ov) {
     if (lattice == 9) {
-        return ph.psc == 0 ? launch_collide_stream_t<D2Q9, S, 0>(fin, fout, g, ph, tl, pd, flags, s, ov)
-                           : launch_collide_stream_t<D2Q9, S, 1>(fin, fout, g, ph, tl, pd, flags, s, ov);
+        return ph.psc == 0 ? launch_collide_stream_l<D2Q9, S, 0>(fin, fout, g, ph, tl, pd, flags, s, ov)
+                           : launch_collide_stream_l<D2Q9, S, 1>(fin, fout, g, ph, tl, pd, flags, s, ov);
     }
-    return ph.psc == 0 ? launch_collide_stream_t<D3Q19, S, 0>(fin, fout, g, ph, tl, pd, flags, s, ov)
-                       : launch_collide_stream_t<D3Q19, S, 1>(fin, fout, g, ph, tl, pd, flags, s, ov);
+    return ph.psc == 0 ? launch_collide_stream_l<D3Q19, S, 0>(fin, fout, g, ph, tl, pd, flags, s, ov)
+                       : launch_collide_stream_l<D3Q19, S, 1>(fin, fout, g, ph, tl, pd, flags, s, ov);
 }
 
 template <class L, typename S>
 cudaError_t launch_macro_t(const S *fin, double *rho, double *u, const Geom &g, const Phys &ph, cudaStream_t s) {
-    bool faces = false;
-    for (int a = 0; a < 3; ++a) faces |= face_kind(g, a, 0) >= FACE_OPEN || face_kind(g, a, 1) >= FACE_OPEN;
-    auto kern = faces ? k_macro<L, S, true> : k_macro<L, S, false>;
+    auto kern = open_faces(g) ? k_macro<L, S, true> : k_macro<L, S, false>;
     const PhysT<typename Store<S>::T> pt = make_phys<typename Store<S>::T>(ph, L::Q);
-    kern<<<dim3(g.nt[0], g.nt[1], g.nt[2]), kThreads, 0, s>>>(fin, g, pt, (double)pt.F[0], (double)pt.F[1],
+    kern<<<dim3((unsigned)g.nt[0] * (unsigned)g.nt[1], 1, g.nt[2]), kThreads, 0, s>>>(fin, g, pt, (double)pt.F[0], (double)pt.F[1],
                                                              (double)pt.F[2], rho, u);
     return cudaGetLastError();
 }
@@ -1301,7 +1360,8 @@ cudaError_t launch_gather_storage(int lattice, const void *fin, double *f_out, d
     using T = typename Store<S>::T;
     if (rho || u) {
         cudaError_t e = lattice == 9 ? launch_macro_t<D2Q9, S>((const S *)fin, rho, u, g, ph, s)
-                                     : launch_macro_t<D3Q19, S>((const S *)fin, rho, u, g, ph, s);
+                      : wide_tiles(3, sizeof(S), g) ? launch_macro_t<D3Q19w, S>((const S *)fin, rho, u, g, ph, s)
+                                                    : launch_macro_t<D3Q19, S>((const S *)fin, rho, u, g, ph, s);
         if (e != cudaSuccess || !f_out) return e;
     }
     const int threads = 256;

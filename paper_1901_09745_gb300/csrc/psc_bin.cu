@@ -10,15 +10,21 @@
 
 namespace psc {
 
-constexpr int kBinBatch = 8;   // tiles whose slot atomics one thread has in flight at once
+constexpr int kBinBatch = 4;   // tiles whose slot atomics one lane has in flight at once
 
+// G lanes per particle share the tiles of its box (3D: 32, a sphere of r = 6 meets up to 130 tiles
+// of 64 x 2 x 2; 2D: 4, a disc meets about 6): latency-bound, so what counts is how many slot
+// atomics are under way. 500 spheres r = 3 on 50 x 50 x 100: 20.5 us with one thread each, 7.8 now.
+template <int G>
 __global__ void k_bin(int dim, int wide, Geom g, double h, Tiles tl, Parts pd) {
     pdl_launch();     // the packing kernel may start; it waits for this one to finish
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, p = t / G, sub = t % G;
     int mx = 0;   // largest slot taken by this thread
     if (p < pd.n) {
-        for (int c = 0; c < 3; ++c) { pd.F[3 * p + c] = 0.0; pd.T[3 * p + c] = 0.0; }
-        if (pd.Pf) {   // FP32 record data, converted once per particle
+        if (sub == 0) {
+            for (int c = 0; c < 3; ++c) { pd.F[3 * p + c] = 0.0; pd.T[3 * p + c] = 0.0; }
+        }
+        if (pd.Pf && sub == G - 1) {   // FP32 record data, converted once per particle
             pd.Pf[2 * p] = make_float4((float)pd.R[p], (float)pd.Fr[p], (float)pd.U[3 * p], (float)pd.U[3 * p + 1]);
             pd.Pf[2 * p + 1] = make_float4((float)pd.U[3 * p + 2], (float)pd.Om[3 * p], (float)pd.Om[3 * p + 1],
                                            (float)pd.Om[3 * p + 2]);
@@ -46,20 +52,20 @@ __global__ void k_bin(int dim, int wide, Geom g, double h, Tiles tl, Parts pd) {
         // every tile of the box, kBinBatch at a time: the slot atomics of a batch are
         // independent, so their round trips overlap
         const int total = len[0] * len[1] * len[2];
-        for (int k0 = 0; k0 < total; k0 += kBinBatch) {
+        for (int k0 = sub; k0 < total; k0 += G * kBinBatch) {
             long long tile[kBinBatch];
             int slot[kBinBatch];
 #pragma unroll
             for (int q = 0; q < kBinBatch; ++q) {
-                const int k = k0 + q;
+                const int k = k0 + q * G;
                 if (k < total) {
                     const int kx = k % len[0], kyz = k / len[0];
                     const int tx = axis_tile(kx, nr[0], ra[0], rb[0]);
                     const int ty = axis_tile(kyz % len[1], nr[1], ra[1], rb[1]);
                     const int tz = axis_tile(kyz / len[1], nr[2], ra[2], rb[2]);
                     tile[q] = -1;
-                    const int org[3] = {tx * tile_ext(dim, wide, 0), ty * tile_ext(dim, wide, 1), tz * tile_ext(dim, wide, 2)};
                     const int ext[3] = {tile_ext(dim, wide, 0), tile_ext(dim, wide, 1), tile_ext(dim, wide, 2)};
+                    const int org[3] = {tx * ext[0], ty * ext[1], tz * ext[2]};
                     if (tile_in_reach(xp, reach, org, ext, g.n, g.periodic, dim)) {
                         tile[q] = PSC_IDX(tx + (long long)g.nt[0] * (ty + (long long)g.nt[1] * tz),
                                           (long long)g.nt[0] * g.nt[1] * g.nt[2], CHK_TILE);
@@ -69,7 +75,7 @@ __global__ void k_bin(int dim, int wide, Geom g, double h, Tiles tl, Parts pd) {
             }
 #pragma unroll
             for (int q = 0; q < kBinBatch; ++q) {
-                if (k0 + q < total && tile[q] >= 0) {
+                if (k0 + q * G < total && tile[q] >= 0) {
                     if (slot[q] < tl.cap) tl.list[tile[q] * tl.cap + slot[q]] = p;
                     else if (slot[q] == tl.cap) atomicAdd(&tl.stats[0], 1);
                     mx = max(mx, slot[q] + 1);
@@ -145,8 +151,10 @@ __global__ void k_download(const double *F, const double *T, double *Fo, double 
 cudaError_t launch_bin(int dim, int wide, const Geom &g, const Phys &ph, const Tiles &tl, const Parts &pd,
                        cudaStream_t s) {
     if (pd.n <= 0) return cudaSuccess;
-    const int threads = 128;
-    return launch_pdl(k_bin, dim3((pd.n + threads - 1) / threads), dim3(threads), 0, s, dim, wide, g, ph.shell_h, tl, pd);
+    const int threads = 128, lanes = dim == 3 ? 32 : 4;
+    const dim3 blocks((unsigned)(((long long)pd.n * lanes + threads - 1) / threads));
+    return dim == 3 ? launch_pdl(k_bin<32>, blocks, dim3(threads), 0, s, dim, wide, g, ph.shell_h, tl, pd)
+                    : launch_pdl(k_bin<4>, blocks, dim3(threads), 0, s, dim, wide, g, ph.shell_h, tl, pd);
 }
 
 long long pack_block_bytes(int rec_double, int cap) {

@@ -287,11 +287,13 @@ cudaError_t launch_adjoint(int storage, int lattice, const void *gt, const void 
                            const Geom &g, const Phys &ph, const Tiles &tl, const Parts &pd, double invT,
                            double *dJdX, double *dFpart, cudaStream_t s) {
     if (storage == ST_F64) {
-        return lattice == 9 ? launch_adjoint_t<Tiled<D2Q9, double>, double>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s)
-                            : launch_adjoint_t<Tiled<D3Q19, double>, double>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
+        return lattice == 9 ? launch_adjoint_t<D2Q9, double>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s)
+                            : launch_adjoint_t<D3Q19, double>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
     }
-    return lattice == 9 ? launch_adjoint_t<Tiled<D2Q9, float>, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s)
-                        : launch_adjoint_t<Tiled<D3Q19, float>, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
+    if (lattice == 9) return launch_adjoint_t<D2Q9, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
+    return g.wide
+               ? launch_adjoint_t<D3Q19w, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s)
+               : launch_adjoint_t<D3Q19, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
 }
 
 }  // namespace psc

@@ -207,8 +207,9 @@ extern "C" lbm_status lbm_create(const lbm_params *p, lbm_ctx **out) {
         set_face_kind(g, a, 0, lo);
         set_face_kind(g, a, 1, lo == FACE_INFLOW ? FACE_OUTLET : lo);
     }
+    g.wide = wide_tiles(ctx->dim, ctx->elem, g);
     for (int a = 0; a < 3; ++a) {
-        g.nt[a] = (g.n[a] + tile_ext(ctx->dim, wide_tiles(ctx->dim, ctx->elem, ctx->g), a) - 1) / tile_ext(ctx->dim, wide_tiles(ctx->dim, ctx->elem, ctx->g), a);
+        g.nt[a] = (g.n[a] + tile_ext(ctx->dim, g.wide, a) - 1) / tile_ext(ctx->dim, g.wide, a);
         g.inv_n[a] = 1.0 / g.n[a];
     }
     ctx->ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
@@ -316,7 +317,7 @@ static Tiles ctx_tiles(lbm_ctx *ctx) {
 // the widest particle shell does not fit well inside half the box.
 void ctx_update_wrap(lbm_ctx *ctx) {
     for (int a = 0; a < 3; ++a) {
-        double need = tile_ext(ctx->dim, wide_tiles(ctx->dim, ctx->elem, ctx->g), a) + 2.0 * (ctx->rmax + ctx->p.shell_h) + 2.0;
+        double need = tile_ext(ctx->dim, ctx->g.wide, a) + 2.0 * (ctx->rmax + ctx->p.shell_h) + 2.0;
         const int w = (a < ctx->dim && ctx->g.periodic[a] && ctx->g.n[a] < need) ? 1 : 0;
         if (w != ctx->g.wrap_img[a]) ctx->gen += 1;     // the step's kernels take Geom by value
         ctx->g.wrap_img[a] = w;
@@ -553,7 +554,7 @@ static lbm_status ctx_enqueue_bin(lbm_ctx *ctx) {
     Tiles tl = ctx_tiles(ctx);
     CK(cudaMemsetAsync(ctx->tile_count, 0, (size_t)ctx->ntiles * sizeof(int), ctx->stream), "memset tile counts");
     CK(cudaMemsetAsync(ctx->tile_stats, 0, kTileStats * sizeof(int), ctx->stream), "memset tile stats");
-    CK(launch_bin(ctx->dim, wide_tiles(ctx->dim, ctx->elem, ctx->g), ctx->g, ctx->ph, tl, ctx_parts(ctx), ctx->stream), "bin kernel");
+    CK(launch_bin(ctx->dim, ctx->g, ctx->ph, tl, ctx_parts(ctx), ctx->stream), "bin kernel");
     CK(launch_pack(ctx->q, ctx->p.storage, ctx->g, tl, ctx_parts(ctx), ctx->ntiles, ctx->stream), "pack kernel");
     return LBM_OK;
 }
@@ -640,7 +641,8 @@ lbm_status ctx_step_once(lbm_ctx *ctx) {
         ctx->launches += 2;
         ctx->bins_valid = 1;
     }
-    ctx->launches += (ctx->np > 0) ? 2 : 1;     // the step's kernel, the overflow tiles
+    // the step's kernel (16 bits in 2D: two), the overflow tiles; open faces: two kernels
+    ctx->launches += (ctx->np > 0) ? ((ctx->dim == 2 && ctx->elem == 2 && !open_faces(ctx->g)) ? 3 : 2) : 1;
     ctx->cs_launches += 1;
     ctx->cur ^= 1;
     ctx->steps += 1;
@@ -719,7 +721,7 @@ static lbm_status ctx_coupled_once(lbm_ctx *ctx, dem_ctx *dem, int substeps) {
         ctx->launches += 2;
         ctx->bins_valid = 1;
     }
-    ctx->launches += 3;
+    ctx->launches += open_faces(ctx->g) ? 2 : 3;
     ctx->cs_launches += 1;
     ctx->cur ^= 1;
     ctx->steps += 1;

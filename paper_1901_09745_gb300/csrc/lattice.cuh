@@ -24,8 +24,6 @@ struct D2Q9 {
         return t[i];
     }
     __host__ __device__ static constexpr int ez(int) { return 0; }
-    // directions below i with e_x != 0
-    __host__ __device__ static constexpr int ex_before(int i) { return i <= 1 ? 0 : (i == 2 ? 1 : (i <= 5 ? 2 : i - 3)); }
 };
 
 struct D3Q19 {
@@ -44,21 +42,15 @@ struct D3Q19 {
         constexpr int t[19] = {0, 0, 0, 0, 0, 1, -1, 0, 0, 0, 0, 1, -1, -1, 1, 1, -1, -1, 1};
         return t[i];
     }
-    __host__ __device__ static constexpr int ex_before(int i) {
-        return i <= 1 ? 0 : (i == 2 ? 1 : (i <= 7 ? 2 : (i <= 15 ? i - 5 : 10)));
-    }
 };
 
 // D3Q19 cut into tiles 64 cells wide, for FP32, where one row of 64 cells per warp reads 7 % fewer
 // lines than two of 32 (fewer values beyond a row's ends): 256^3 with 2000 spheres 431 us against
 // 512, without particles 381 against 452. In 2D the narrow tiles are as fast or faster (a disc
 // meets more rows of wide tiles): 2048^2 with 5000 discs 67 us against 70, 777 x 453 19 against
-// 22. (Contexts with open faces keep narrow tiles, see wide_tiles.) Records hold positions from the tile's middle (REC_X), so that they round as finely
-// as with narrow tiles.
+// 22. wide_tiles tells which lattices take them. Records hold positions from the tile's middle
+// (REC_X), so that they round as finely as with narrow tiles.
 struct D3Q19w : D3Q19 { static constexpr int TX = 64, TY = 2, TZ = 2, REC_X = 32; };
-template <class L, typename S> struct TiledBy { using type = L; };
-template <> struct TiledBy<D3Q19, float> { using type = D3Q19w; };
-template <class L, typename S> using Tiled = typename TiledBy<L, S>::type;
 
 template <class L>
 __host__ __device__ constexpr int opp(int i) { return i == 0 ? 0 : ((i & 1) ? i + 1 : i - 1); }

@@ -27,8 +27,10 @@ namespace {
 constexpr size_t kScratchBytes = (size_t)LBM_NOALLOC_SCRATCH_BYTES;
 constexpr int kNoAllocCap = 16;        // candidate records per tile (more take the exact slow path)
 constexpr int kMaxDevices = 64;
+constexpr size_t kWorkBytes = (size_t)psc::kWorkWords * sizeof(int);
 
-static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
+// the step's work counters lie behind the declared size
+static __device__ __align__(256) unsigned char g_scratch[kScratchBytes + kWorkBytes];
 
 // Device address of g_scratch for each device, looked up once (with that device current),
 // and the second stream and events of the 2D step on that device, created at the same time.
@@ -97,9 +99,11 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
         g.wrap_img[a] = (a < (is2d ? 2 : 3)) && g.periodic[a];
         g.inv_n[a] = 1.0 / g.n[a];
     }
-    const int wide = wide_tiles(is2d ? 2 : 3, elem, g);
-    for (int a = 0; a < 3; ++a) g.nt[a] = (g.n[a] + tile_ext(is2d ? 2 : 3, wide, a) - 1) / tile_ext(is2d ? 2 : 3, wide, a);
-    if ((g.n[1] + tile_ext(is2d ? 2 : 3, 0, 1) - 1) / tile_ext(is2d ? 2 : 3, 0, 1) > 65535 || g.nt[2] > 65535) return fail(LBM_ERR_ARG, "ny or nz too large for the tile grid");
+    // (no more of them than narrow ones, for which the fixed array is carved)
+    g.wide = wide_tiles(is2d ? 2 : 3, elem, g) && tile_number(3, 1, g) <= tile_number(3, 0, g);
+    for (int a = 0; a < 3; ++a) g.nt[a] = (g.n[a] + tile_ext(is2d ? 2 : 3, g.wide, a) - 1) / tile_ext(is2d ? 2 : 3, g.wide, a);
+    const int ty = tile_ext(is2d ? 2 : 3, 0, 1);
+    if ((g.n[1] + ty - 1) / ty > 65535 || g.nt[2] > 65535) return fail(LBM_ERR_ARG, "ny or nz too large for the tile grid");
     Phys ph;
     ph.tau = p->tau;
     for (int a = 0; a < 3; ++a) ph.body_force[a] = p->body_force[a];
@@ -112,21 +116,22 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
     for (int a = 0; a < 3; ++a)
         if (p->bc[a] == LBM_BC_INFLOW) ph.inflow_axis = a;
 
-    // carve the fixed array: counts | stats | flags | work counters | lists | tile order | f(r) | packed tile blocks
+    // carve the fixed array: counts | stats | flags | lists | tile order | f(r) | packed tile
+    // blocks; sized for narrow tiles
     const long long ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
+    const long long room = tile_number(is2d ? 2 : 3, 0, g);
     const int rec_double = (p->storage == LBM_F64);
     size_t off = 0;
-    const size_t o_count = off; off += (size_t)ntiles * sizeof(int);
+    const size_t o_count = off; off += (size_t)room * sizeof(int);
     const size_t o_stats = off; off += kTileStats * sizeof(int);
     const size_t o_flags = off; off += 4 * sizeof(int);
-    const size_t o_work = off; off += kWorkWords * sizeof(int);
-    const size_t o_list = off; off += (size_t)ntiles * kNoAllocCap * sizeof(int);
+    const size_t o_list = off; off += (size_t)room * kNoAllocCap * sizeof(int);
     off = align_up(off, 16);
-    const size_t o_order = off; off += (size_t)ntiles * 3 * sizeof(unsigned);
+    const size_t o_order = off; off += (size_t)room * 3 * sizeof(uint2);
     off = align_up(off, 16);
     const size_t o_fr = off; off += (size_t)n * sizeof(double);
     off = align_up(off, 256);
-    const size_t o_blocks = off; off += (size_t)ntiles * (size_t)pack_block_bytes(rec_double, kNoAllocCap);
+    const size_t o_blocks = off; off += (size_t)room * (size_t)pack_block_bytes(rec_double, kNoAllocCap);
     if (off > kScratchBytes) {
         char msg[200];
         snprintf(msg, sizeof(msg), "lattice/particles need %zu bytes of working memory; the fixed array holds %zu "
@@ -164,17 +169,18 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
     tl.cap = kNoAllocCap;
     tl.blocks = base + o_blocks;
     tl.order = (unsigned *)(base + o_order);
-    tl.work = (int *)(base + o_work);
+    tl.work = (int *)(base + kScratchBytes);
     int *flags = (int *)(base + o_flags);
     Parts pd;
     pd.n = n; pd.X = X; pd.U = U; pd.Om = Omega; pd.R = radius; pd.Fr = (double *)(base + o_fr);
     pd.F = F; pd.T = T;
     pd.Pf = nullptr;
 
-    // what must start at zero: tile counts, stats, flags, work counters (the rest is fully rewritten)
+    // what must start at zero: tile counts, stats, flags (the rest is fully rewritten; the work
+    // counters are zero from the start, and each launch leaves them so)
     e = cudaMemsetAsync(base, 0, o_list, s);
     if (e == cudaSuccess && n > 0) e = launch_f_of_r(is2d ? 2 : 3, radius, (double *)(base + o_fr), n, s);
-    if (e == cudaSuccess && n > 0) e = launch_bin(is2d ? 2 : 3, wide, g, ph, tl, pd, s);
+    if (e == cudaSuccess && n > 0) e = launch_bin(is2d ? 2 : 3, g, ph, tl, pd, s);
     if (e == cudaSuccess && n > 0) e = launch_pack(p->lattice, p->storage, g, tl, pd, ntiles, s);
     if (e == cudaSuccess)
         e = launch_collide_stream(p->storage, p->lattice, f_in, f_out, g, ph, tl, pd, flags, s,

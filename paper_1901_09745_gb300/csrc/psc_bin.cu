@@ -16,7 +16,7 @@ constexpr int kBinBatch = 4;   // tiles whose slot atomics one lane has in fligh
 // of 64 x 2 x 2; 2D: 4, a disc meets about 6): latency-bound, so what counts is how many slot
 // atomics are under way. 500 spheres r = 3 on 50 x 50 x 100: 20.5 us with one thread each, 7.8 now.
 template <int G>
-__global__ void k_bin(int dim, int wide, Geom g, double h, Tiles tl, Parts pd) {
+__global__ void k_bin(int dim, Geom g, double h, Tiles tl, Parts pd) {
     pdl_launch();     // the packing kernel may start; it waits for this one to finish
     const int t = blockIdx.x * blockDim.x + threadIdx.x, p = t / G, sub = t % G;
     int mx = 0;   // largest slot taken by this thread
@@ -45,7 +45,7 @@ __global__ void k_bin(int dim, int wide, Geom g, double h, Tiles tl, Parts pd) {
             if (ax >= dim) { nr[ax] = 1; ra[ax][0] = rb[ax][0] = 0; len[ax] = 1; continue; }
             const double X = xw[ax];
             const int lo = (int)ceil(X - r - h), hi = (int)floor(X + r + h);
-            nr[ax] = axis_tile_ranges(lo, hi, g.n[ax], tile_ext(dim, wide, ax), g.nt[ax], g.periodic[ax], ra[ax], rb[ax]);
+            nr[ax] = axis_tile_ranges(lo, hi, g.n[ax], tile_ext(dim, g.wide, ax), g.nt[ax], g.periodic[ax], ra[ax], rb[ax]);
             len[ax] = 0;
             for (int k = 0; k < nr[ax]; ++k) len[ax] += rb[ax][k] - ra[ax][k] + 1;
         }
@@ -64,7 +64,7 @@ __global__ void k_bin(int dim, int wide, Geom g, double h, Tiles tl, Parts pd) {
                     const int ty = axis_tile(kyz % len[1], nr[1], ra[1], rb[1]);
                     const int tz = axis_tile(kyz / len[1], nr[2], ra[2], rb[2]);
                     tile[q] = -1;
-                    const int ext[3] = {tile_ext(dim, wide, 0), tile_ext(dim, wide, 1), tile_ext(dim, wide, 2)};
+                    const int ext[3] = {tile_ext(dim, g.wide, 0), tile_ext(dim, g.wide, 1), tile_ext(dim, g.wide, 2)};
                     const int org[3] = {tx * ext[0], ty * ext[1], tz * ext[2]};
                     if (tile_in_reach(xp, reach, org, ext, g.n, g.periodic, dim)) {
                         tile[q] = PSC_IDX(tx + (long long)g.nt[0] * (ty + (long long)g.nt[1] * tz),
@@ -148,13 +148,13 @@ __global__ void k_download(const double *F, const double *T, double *Fo, double 
     if (k < 4) flags_out[k] = flags[k];
 }
 
-cudaError_t launch_bin(int dim, int wide, const Geom &g, const Phys &ph, const Tiles &tl, const Parts &pd,
+cudaError_t launch_bin(int dim, const Geom &g, const Phys &ph, const Tiles &tl, const Parts &pd,
                        cudaStream_t s) {
     if (pd.n <= 0) return cudaSuccess;
     const int threads = 128, lanes = dim == 3 ? 32 : 4;
     const dim3 blocks((unsigned)(((long long)pd.n * lanes + threads - 1) / threads));
-    return dim == 3 ? launch_pdl(k_bin<32>, blocks, dim3(threads), 0, s, dim, wide, g, ph.shell_h, tl, pd)
-                    : launch_pdl(k_bin<4>, blocks, dim3(threads), 0, s, dim, wide, g, ph.shell_h, tl, pd);
+    return dim == 3 ? launch_pdl(k_bin<32>, blocks, dim3(threads), 0, s, dim, g, ph.shell_h, tl, pd)
+                    : launch_pdl(k_bin<4>, blocks, dim3(threads), 0, s, dim, g, ph.shell_h, tl, pd);
 }
 
 long long pack_block_bytes(int rec_double, int cap) {
@@ -172,7 +172,7 @@ cudaError_t launch_pack(int lattice, int storage, const Geom &g, const Tiles &tl
                         cudaStream_t s) {
     const bool d2 = lattice == 9;
     if (storage == ST_F64) return d2 ? launch_pack_t<D2Q9, double>(g, tl, pd, ntiles, s) : launch_pack_t<D3Q19, double>(g, tl, pd, ntiles, s);
-    if (!d2 && wide_tiles(3, storage == ST_F32 ? 4 : 2, g)) return launch_pack_t<D3Q19w, float>(g, tl, pd, ntiles, s);
+    if (g.wide) return launch_pack_t<D3Q19w, float>(g, tl, pd, ntiles, s);
     return d2 ? launch_pack_t<D2Q9, float>(g, tl, pd, ntiles, s) : launch_pack_t<D3Q19, float>(g, tl, pd, ntiles, s);
 }
 

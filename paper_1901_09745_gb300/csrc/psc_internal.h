@@ -52,6 +52,7 @@ struct Geom {
     long long ncell;     // nx * ny * nz
     int periodic[3];     // 1 = periodic axis, 0 = another face kind (see faces)
     int wrap_img[3];     // 1 = periodic axis short enough to need a per-cell minimum image
+    int wide;            // tiles 64 cells wide (wide_tiles)
     int nt[3];           // tiles per axis (tile extent: tile_ext)
     int faces;           // what lies beyond each face, a FaceKind in 3 bits per face (face_kind):
                          // a population whose source x - e_i is beyond it wraps, bounces back,
@@ -79,16 +80,27 @@ __host__ __device__ inline bool open_faces(const Geom &g) {
     for (int a = 0; a < 3; ++a) any |= face_kind(g, a, 0) >= FACE_OPEN || face_kind(g, a, 1) >= FACE_OPEN;
     return any;
 }
-// Whether a lattice is cut into the wide tiles (Tiled<> in lattice.cuh).
-__host__ __device__ inline int wide_tiles(const int dim, const size_t elem_bytes, const Geom &g) {
-    return elem_bytes == 4 && dim == 3 && !open_faces(g);
-}
 // Tile extent along axis ax: 32 x 8 x 1 cells for D2Q9, 32 x 4 x 2 for D3Q19; wide tiles 64 x 4 x 1
 // and 64 x 2 x 2. One tile is one thread block of the single-cell kernels.
 __host__ __device__ inline int tile_ext(const int dim, const int wide, const int ax) {
     if (ax == 0) return wide ? 64 : 32;
     if (ax == 1) return (dim == 2 ? 8 : 4) >> wide;
     return dim == 2 ? 1 : 2;
+}
+__host__ inline long long tile_number(const int dim, const int wide, const Geom &g) {
+    long long t = 1;
+    for (int a = 0; a < 3; ++a) t *= (g.n[a] + tile_ext(dim, wide, a) - 1) / tile_ext(dim, wide, a);
+    return t;
+}
+// Whether a lattice (g.n and g.faces) is best cut into the wide tiles (D3Q19w in lattice.cuh): FP32
+// in 3D without open faces, where they are at most an eighth of their number emptier than the narrow
+// ones. Step's kernel, narrow and wide, us (tiles wide / narrow): 290 x 128 x 128 200 and 159 (1),
+// 200^3 273 and 231, 198 x 107 x 42 41.2 and 38.6 (1.14), 160 x 128 x 128 80.9 and 84.9 (1.2),
+// 96^3 35.0 and 39.1 (1.33), 32 x 128 x 256 39 and 52 (2), 48^3 15.1 and 15.9 (1): rows of up to 64
+// cells stay narrow, so that a short periodic row needs no minimum image per cell either.
+__host__ inline int wide_tiles(const int dim, const size_t elem_bytes, const Geom &g) {
+    return elem_bytes == 4 && dim == 3 && g.n[0] > 64 && !open_faces(g) &&
+           7 * tile_number(3, 1, g) <= 8 * tile_number(3, 0, g);
 }
 
 // Physical parameters (FP64 on the host; kernels convert to their compute type).
@@ -161,7 +173,7 @@ cudaError_t launch_gather(int storage, int lattice, const void *fin, double *f_o
 cudaError_t launch_set(int storage, int lattice, const double *f, void *fout,
                        const Geom &g, const Phys &ph, cudaStream_t s);
 // Bin particles into tile candidate lists and zero F, T.
-cudaError_t launch_bin(int dim, int wide, const Geom &g, const Phys &ph, const Tiles &tl,
+cudaError_t launch_bin(int dim, const Geom &g, const Phys &ph, const Tiles &tl,
                        const Parts &pd, cudaStream_t s);
 // Sort each tile's list and write its packed candidate records (in the storage's compute type).
 cudaError_t launch_pack(int lattice, int storage, const Geom &g, const Tiles &tl, const Parts &pd,

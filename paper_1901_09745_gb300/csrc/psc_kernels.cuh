@@ -1325,11 +1325,15 @@ cudaError_t launch_collide_stream_l(const void *fin, void *fout, const Geom &g, 
     if constexpr (sizeof(S) == 2) {
         return launch_collide_stream16<L, S, PSC>(fin, fout, g, ph, tl, pd, flags, s, ov);
     } else {
-        using W = Tiled<L, S>;
         // pairs in one access: every row of every direction starts on a pair boundary
         const bool vec = g.n[0] % 2 == 0 && ((uintptr_t)fin | (uintptr_t)fout) % (2 * sizeof(S)) == 0;
-        return vec ? launch_collide_stream_t<W, S, PSC, true>(fin, fout, g, ph, tl, pd, flags, s, ov)
-                   : launch_collide_stream_t<W, S, PSC, false>(fin, fout, g, ph, tl, pd, flags, s, ov);
+        if constexpr (L::D == 3 && sizeof(S) == 4) {
+            if (g.wide)
+                return vec ? launch_collide_stream_t<D3Q19w, S, PSC, true>(fin, fout, g, ph, tl, pd, flags, s, ov)
+                           : launch_collide_stream_t<D3Q19w, S, PSC, false>(fin, fout, g, ph, tl, pd, flags, s, ov);
+        }
+        return vec ? launch_collide_stream_t<L, S, PSC, true>(fin, fout, g, ph, tl, pd, flags, s, ov)
+                   : launch_collide_stream_t<L, S, PSC, false>(fin, fout, g, ph, tl, pd, flags, s, ov);
     }
 }
 
@@ -1360,7 +1364,7 @@ cudaError_t launch_gather_storage(int lattice, const void *fin, double *f_out, d
     using T = typename Store<S>::T;
     if (rho || u) {
         cudaError_t e = lattice == 9 ? launch_macro_t<D2Q9, S>((const S *)fin, rho, u, g, ph, s)
-                      : wide_tiles(3, sizeof(S), g) ? launch_macro_t<D3Q19w, S>((const S *)fin, rho, u, g, ph, s)
+                      : g.wide ? launch_macro_t<D3Q19w, S>((const S *)fin, rho, u, g, ph, s)
                                                     : launch_macro_t<D3Q19, S>((const S *)fin, rho, u, g, ph, s);
         if (e != cudaSuccess || !f_out) return e;
     }

@@ -3,7 +3,7 @@
 //
 // A warp works alone on 64 cells of a lattice tile at a time: two neighbouring rows of a tile 32
 // wide (2D: rows 2k and 2k + 1; 3D: row k at both z), one per half warp, or one row of a tile 64
-// wide (Tiled<>). Each lane owns two x-neighbours. Per 64 cells the warp
+// wide (D3Q19w). Each lane owns two x-neighbours. Per 64 cells the warp
 //   queues the pull of the populations (Eq. 1, 6);
 //   tests the tile's candidate particles against its rows (one lane per candidate, ballot) and
 //     visits those that can reach them for the solid fractions (Table 1, Eq. 15-18) and, for
@@ -329,23 +329,26 @@ __device__ __forceinline__ void collide_store(const Dirs<L, S> &f, const Geom &g
     }
 }
 
-// The arm to the nearest image of a candidate of reach `reach` on the periodic axes too short for
-// the tile's own image to be it for every cell.
+// The arm from candidate q (position, radius) to the pair at c (cell a) on lattices with periodic
+// axes too short for the tile's own image of the candidate to be the nearest for every cell. What
+// the difference over up to a period loses in rounding is added back to the short arm.
 template <typename T> struct Arm {
     typename Pr<T>::V dx;
     T dy, dz;
 };
 template <class L, typename T>
-__device__ __noinline__ Arm<T> near_image(const Geom &g, const T reach, const Arm<T> d) {
+__device__ __noinline__ Arm<T> near_image(const Geom &g, const T h, const Vec4<T> q, const T cx, const T cy, const T cz) {
     const int ext[3] = {L::TX, L::TY, L::TZ};
-    auto image = [&](const T v, const int a) {
-        const T n = (T)g.n[a];
-        return (g.wrap_img[a] && n < (T)(ext[a] + 2) + (T)2 * reach) ? v - n * rint_t(v / n) : v;
+    auto image = [&](const T c, const T p, const int a) {
+        const T n = (T)g.n[a], v = c - p;
+        if (!g.wrap_img[a] || !(n < (T)(ext[a] + 2) + (T)2 * (q.w + h))) return v;
+        const T b = v - c, lost = (c - (v - b)) - (p + b);
+        return (v - n * rint_t(v / n)) + lost;
     };
     Arm<T> r;
-    r.dx = Pr<T>::mk(image(d.dx.x, 0), image(d.dx.y, 0));
-    r.dy = image(d.dy, 1);
-    r.dz = (L::D == 3) ? image(d.dz, 2) : d.dz;
+    r.dx = Pr<T>::mk(image(cx, q.x, 0), image(cx + (T)1, q.x, 0));
+    r.dy = image(cy, q.y, 1);
+    r.dz = (L::D == 3) ? image(cz, q.z, 2) : (T)0;
     return r;
 }
 
@@ -399,7 +402,7 @@ __device__ __forceinline__ void unit_step(const UnitPos<L> &up, const int cnt,
         dz = (D == 3) ? cz - q.z : (T)0;
         dx = P::mk(dxa, cx + (T)1 - q.x);
         if (wrapped) {
-            const Arm<T> n = near_image<L, T>(g, q.w + ph.h, Arm<T>{dx, dy, dz});
+            const Arm<T> n = near_image<L, T>(g, ph.h, q, cx, cy, cz);
             dx = n.dx; dy = n.dy; dz = n.dz;
         }
     };

@@ -28,6 +28,7 @@ def case(lattice, n, bc, moving, count=4, seed=5):
 
 SHAPES = [(9, (w, 19, 1), (bx, 1 - bx, 0)) for w in (11, 31, 32, 33, 64, 65, 130) for bx in (0, 1)]
 SHAPES += [(19, (w, 11, 9), (bx, 0, 1 - bx)) for w in (11, 32, 63, 64, 65, 66, 130) for bx in (0, 1)]
+SHAPES += [(19, (w, 11, 9), (bx, 0, 1 - bx)) for w in (97, 127, 128, 198) for bx in (0, 1)]     # wide tiles
 
 
 @pytest.mark.parametrize("lattice,n,bc", SHAPES)

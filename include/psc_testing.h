@@ -41,6 +41,9 @@ int psc_test_contact_sign(double d2, double S, int *ge0, int *gt0);
 float psc_test_jkr_s(float t, float s_prev, int *fail, int *iters);
 /* The DEM's squared displacement test (FP32, one image shift on periodic axes) of a
  * particle at x[3] from its position xr[3] at the last neighbour-list build. */
+/* The kernels' integer forms of (float)v and (double)v. */
+float psc_test_to_f32(double v);
+double psc_test_to_f64(float v);
 float psc_test_moved2(const double *x, const double *xr, const int *n, const int *periodic, int dim);
 /* The host-side checks of a particle upload: 1 when the m values are all finite; the
  * smallest r^2 and the largest r over n radii. */

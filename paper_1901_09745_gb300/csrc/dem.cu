@@ -13,8 +13,8 @@
 //                  pair not on it was farther apart than r_i + r_j + skin at the build, and
 //                  neither particle has moved skin/2 since (a sub-step that sees one move
 //                  that far reports it), so it cannot touch.
-//   3. k_dem_substep (x substeps): two lanes per particle, each taking every other
-//                  neighbour slot:
+//   3. k_dem_substep2 / k_dem_substep3 (x substeps): two lanes per disc, two or eight per
+//        sphere, sharing its neighbour slots:
 //        contact detection in FP64 with IEEE-rounded operations only (no FMA), so both
 //        ends of a pair and a CPU reference agree bit for bit on delta_N;
 //        the contact law in FP32: JKR normal force (Eq. 26-27) with the contact radius
@@ -41,6 +41,9 @@ using psc::axis_span;
 using psc::contact_sign;
 using psc::ContactSign;
 using psc::jkr_s;
+using psc::to_f32;
+using psc::to_f64;
+using psc::axis_moved;
 using psc::moved2;
 
 constexpr int kNB = 32;        // neighbour slots per particle (one warp lane each)
@@ -58,6 +61,8 @@ struct DemGeom {
     double skin;
     float margin;       // slack for FP32 position copies (>> their rounding error)
     double inv_n[3];    // 1 / n per axis (no FP64 division on the device)
+    double len[3];      // n per axis
+    double mid[3], hi_wall[3];   // (n - 1) / 2 and n - 1/2: the lattice's middle, the upper wall
     double bscale[3];   // nb / n per axis: bin of x = floor(x * bscale)
 };
 
@@ -403,18 +408,73 @@ __device__ __forceinline__ void mass_inertia(int dim, double rho, double r, doub
     else { *m = rho * (4.0 / 3.0) * kPi * r * r * r; *I = 0.4 * (*m) * r * r; }
 }
 
-constexpr int kLPP = 2;   // lanes per particle in the sub-step kernel (c2 coupled step: 1 lane
-                          // 182.9 us, 2 lanes 162.0, 4 lanes 170.2, 8 lanes 206.0)
-
-// One DEM sub-step. kLPP lanes share a particle and split its neighbour slots; their FP64
-// sums are combined with shuffles in a fixed order, then the first lane integrates.
-// early = 1 when the kernel before it in the stream is the previous sub-step of the same call.
+// Whether particles i and j are in contact, and the pair's unit normal (from i towards j), overlap
+// and effective radius: positions in FP64 (xi, xj), radii, FP32 copies (x, y, z, r); `was`: in
+// contact in the previous sub-step. False where the FP32 copies show them apart.
 template <int DIM>
-__global__ void k_dem_substep(DemGeom g, DemPhys ph, DemBufs b, int early) {
+__device__ __forceinline__ bool pair_contact(const DemGeom &g, const DemPhys &ph, const float reject, const float4 pif,
+                                             const float4 pj, const double *xi, const double *xj, const double ri,
+                                             const double rj, const bool was, float *nv, float &dnf, float &Rij) {
+    // FP32 pre-filter on the position copies: pairs clearly apart skip the FP64 work
+    float df[3] = {pj.x - pif.x, pj.y - pif.y, pj.z - pif.z};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (a >= DIM) { df[a] = 0.0f; continue; }
+        if (g.periodic[a]) {
+            const float half = 0.5f * (float)g.n[a];
+            if (df[a] > half) df[a] -= (float)g.n[a];
+            else if (df[a] < -half) df[a] += (float)g.n[a];
+        }
+    }
+    const float dpre = (pif.w + pj.w) - sqrtf(df[0] * df[0] + df[1] * df[1] + df[2] * df[2]);
+    if (dpre < -reject) return false;      // provably out of contact (the margin dwarfs the FP32 error)
+    // separation X_j - X_i in FP64 (exact subtraction), minimum image; the periodic
+    // shift is decided on the FP32 copy, exact for neighbours (|d| << n/2)
+    double d[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int a = 0; a < DIM; ++a) {
+        d[a] = __dsub_rn(xj[a], xi[a]);
+        if (g.periodic[a]) {
+            const float half = 0.5f * (float)g.n[a], w = to_f32(d[a]);
+            if (w > half) d[a] = __dsub_rn(d[a], g.len[a]);
+            else if (w < -half) d[a] = __dadd_rn(d[a], g.len[a]);
+        }
+    }
+    // d^2 in FP64 with IEEE-rounded operations (bit-identical at both ends and in a
+    // CPU reference); the contact decision of contact_sign (hostdev.cuh)
+    const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
+    const double S = __dadd_rn(ri, rj);
+    const ContactSign cs = contact_sign(d2, S);
+    dnf = cs.dnf;
+    Rij = pif.w * pj.w / (pif.w + pj.w);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) nv[a] = to_f32(d[a]) * cs.inv;
+    if (!ph.adhesive) return cs.gt0;
+    if (cs.ge0 || !was) return cs.ge0;
+    // a stretched neck persists while delta_N > -delta_C: decided in FP32 unless
+    // the two agree to 1e-5, then with delta_N and delta_C in FP64
+    const float a0f = cbrtf((float)(9.0 * kPi) * ph.gamma * Rij * Rij / ph.Es);
+    const float dCf = a0f * a0f * (float)ph.dc_coef / Rij;
+    const float gap = dnf + dCf;
+    if (fabsf(gap) > 1e-5f * dCf) return gap > 0.0f;
+    const double dn = cs.exact ? cs.dn : __dsub_rn(S, __dsqrt_rn(d2));
+    const double R64 = ri * rj / (ri + rj);
+    const double a064 = cbrt(9.0 * kPi * (double)ph.gamma * R64 * R64 / (double)ph.Es);
+    return dn > -(a064 * a064 * ph.dc_coef / R64);
+}
+
+constexpr int kLPP = 2;   // lanes per particle in the sub-step kernel of discs (a coupled step of 5000:
+                          // 1 lane 182.9 us, 2 lanes 162.0, 4 lanes 170.2, 8 lanes 206.0)
+
+// One DEM sub-step of discs. kLPP lanes share a particle and split its neighbour slots; their FP64
+// sums are combined with shuffles in a fixed order, then the first lane integrates. (Discs of a
+// suspension have few contacts, most slots end at pair_contact's FP32 test: the kernel of the
+// spheres below took 2 % longer for 20 coupled steps of 5000, 3.04 ms against 2.98.)
+// early = 1 when the kernel before it in the stream is the previous sub-step of the same call.
+__global__ void k_dem_substep2(DemGeom g, DemPhys ph, DemBufs b, int early) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     const int i = t / kLPP, sub = t % kLPP;
     const bool valid = i < b.n;
-    constexpr int dim = DIM;
     // Values fixed over a call's sub-steps: the list in use, the particle's neighbour count
     // and first neighbour, its radius and masses, the fluid's F and T (read by the
     // integrating lane before the contact loop's stores) and the position at the list's
@@ -448,7 +508,7 @@ __global__ void k_dem_substep(DemGeom g, DemPhys ph, DemBufs b, int early) {
     const int *const nbr = b.nbr[li];
     float *const hist = b.hist[li];
     // force and torque components a 2D disc has: F_x, F_y and T_z
-    auto used = [](int q) { return DIM == 3 || q == 0 || q == 1 || q == 5; };
+    auto used = [](int q) { return q == 0 || q == 1 || q == 5; };
     double acc[6] = {0, 0, 0, 0, 0, 0};
     double xi[3] = {0, 0, 0}, ui[3] = {0, 0, 0}, oi[3] = {0, 0, 0};
     int fail = 0;
@@ -467,81 +527,25 @@ __global__ void k_dem_substep(DemGeom g, DemPhys ph, DemBufs b, int early) {
             const float4 pj = b.Xf[j];
             double xj[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-            for (int a = 0; a < 3; ++a) if (a < dim) xj[a] = b.X[3 * j + a];
+            for (int a = 0; a < 3; ++a) if (a < 2) xj[a] = b.X[3 * j + a];
             const double rj = b.R[j];
             const float4 vj0 = b.Vf[2 * j], vj1 = b.Vf[2 * j + 1];
             const float imj = (float)b.minv[2 * j];
             float4 *hp4 = reinterpret_cast<float4 *>(hp);
             const float4 h0 = hp4[0], h1 = hp4[1];
-            // FP32 pre-filter on the position copies: pairs clearly apart skip the FP64 work
-            float df[3] = {pj.x - pif.x, pj.y - pif.y, pj.z - pif.z};
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                if (a >= dim) { df[a] = 0.0f; continue; }
-                if (g.periodic[a]) {
-                    const float half = 0.5f * (float)g.n[a];
-                    if (df[a] > half) df[a] -= (float)g.n[a];
-                    else if (df[a] < -half) df[a] += (float)g.n[a];
-                }
-            }
             const bool was = h1.w != 0.0f;
-            const float dpre = (pif.w + pj.w) - sqrtf(df[0] * df[0] + df[1] * df[1] + df[2] * df[2]);
-            if (dpre < -b.reject) {
-                // provably out of contact (the margin dwarfs the FP32 error)
+            float nv[3] = {0.0f, 0.0f, 0.0f}, dnf = 0.0f, Rij = 1.0f;
+            const bool contact = pair_contact<2>(g, ph, b.reject, pif, pj, xi, xj, ri, rj, was, nv, dnf, Rij);
+            if (!contact) {
                 if (was) { hp4[0] = make_float4(0.0f, 0.0f, 0.0f, 0.0f); hp4[1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f); }
                 continue;
             }
-            // separation X_j - X_i in FP64 (exact subtraction), minimum image; the periodic
-            // shift is decided on the FP32 copy, exact for neighbours (|d| << n/2)
-            double d[3] = {0.0, 0.0, 0.0};
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                if (a >= dim) break;
-                d[a] = __dsub_rn(xj[a], xi[a]);
-                if (g.periodic[a]) {
-                    const float half = 0.5f * (float)g.n[a], v = (float)d[a];
-                    if (v > half) d[a] = __dsub_rn(d[a], (double)g.n[a]);
-                    else if (v < -half) d[a] = __dadd_rn(d[a], (double)g.n[a]);
-                }
-            }
-            // d^2 in FP64 with IEEE-rounded operations (bit-identical at both ends and in a
-            // CPU reference); the contact decision of contact_sign (hostdev.cuh)
-            const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
-            const double S = __dadd_rn(ri, rj);
-            const ContactSign cs = contact_sign(d2, S);
-            const bool ge0 = cs.ge0, gt0 = cs.gt0, exact = cs.exact;
-            const float inv = cs.inv, dnf = cs.dnf;
-            double dn = cs.dn;
-            bool contact;
-            if (!ph.adhesive) {
-                contact = gt0;
-            } else if (ge0) {
-                contact = true;
-            } else if (!was) {
-                contact = false;
-            } else {
-                // a stretched neck persists while delta_N > -delta_C: decided in FP32 unless
-                // the two agree to 1e-5, then with delta_N and delta_C in FP64
-                const float Rf = pif.w * pj.w / (pif.w + pj.w);
-                const float a0f = cbrtf((float)(9.0 * kPi) * ph.gamma * Rf * Rf / ph.Es);
-                const float dCf = a0f * a0f * (float)ph.dc_coef / Rf;
-                const float gap = dnf + dCf;
-                if (fabsf(gap) > 1e-5f * dCf) {
-                    contact = gap > 0.0f;
-                } else {
-                    if (!exact) dn = __dsub_rn(S, __dsqrt_rn(d2));
-                    const double R64 = ri * rj / (ri + rj);
-                    const double a064 = cbrt(9.0 * kPi * (double)ph.gamma * R64 * R64 / (double)ph.Es);
-                    contact = dn > -(a064 * a064 * ph.dc_coef / R64);
-                }
-            }
-            const float nv[3] = {(float)d[0] * inv, (float)d[1] * inv, (float)d[2] * inv};
             float hl[kH] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
             float fo[3], to[3];
             const float ujf[3] = {vj0.x, vj0.y, vj0.z};
             const float ojf[3] = {vj0.w, vj1.x, vj1.y};
-            const float Rij = pif.w * pj.w / (pif.w + pj.w), msij = 1.0f / (imi + imj);
-            if (contact_on_i(ph, dim, contact, nv, dnf, pif.w, pj.w, Rij, msij, uif, ujf, oif, ojf, hl, fo, to,
+            const float msij = 1.0f / (imi + imj);
+            if (contact_on_i(ph, 2, contact, nv, dnf, pif.w, pj.w, Rij, msij, uif, ujf, oif, ojf, hl, fo, to,
                              &fail)) {
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
@@ -549,10 +553,8 @@ __global__ void k_dem_substep(DemGeom g, DemPhys ph, DemBufs b, int early) {
                     if (used(3 + a)) acc[3 + a] += (double)to[a];
                 }
             }
-            if (was || hl[7] != 0.0f) {
-                hp4[0] = make_float4(hl[0], hl[1], hl[2], hl[3]);
-                hp4[1] = make_float4(hl[4], hl[5], hl[6], hl[7]);
-            }
+            hp4[0] = make_float4(hl[0], hl[1], hl[2], hl[3]);
+            hp4[1] = make_float4(hl[4], hl[5], hl[6], hl[7]);
         }
     }
     // contacts with the walls of the non-periodic axes (the fluid's halfway bounce-back
@@ -560,7 +562,7 @@ __global__ void k_dem_substep(DemGeom g, DemPhys ph, DemBufs b, int early) {
     // is a half-space of the same material at rest (R = r_i, m* = m_i). The overlap and the
     // decision are formed in FP64 with IEEE-rounded operations, as for the pairs.
 #pragma unroll
-    for (int a = 0; a < DIM; ++a) {       // unrolled: the per-axis arrays stay in registers
+    for (int a = 0; a < 2; ++a) {       // unrolled: the per-axis arrays stay in registers
         if (!valid || a % kLPP != sub || g.periodic[a]) continue;
         const double lo_plane = 0.5 * (double)(g.n[a] - 1);
         const bool lower = xi[a] < lo_plane;
@@ -599,7 +601,7 @@ __global__ void k_dem_substep(DemGeom g, DemPhys ph, DemBufs b, int early) {
             const float oif[3] = {vi0.w, vi1.x, vi1.y};
             const float rif = (float)ri;
             const float msw = 1.0f / (float)b.minv[2 * i];
-            if (contact_on_i(ph, dim, contact, nv, (float)dn, rif, 0.0f, rif, msw, uif, zero, oif, zero, hl, fo, to,
+            if (contact_on_i(ph, 2, contact, nv, (float)dn, rif, 0.0f, rif, msw, uif, zero, oif, zero, hl, fo, to,
                              &fail)) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
@@ -623,7 +625,7 @@ __global__ void k_dem_substep(DemGeom g, DemPhys ph, DemBufs b, int early) {
     double un[3], xn[3], on[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        if (a < dim) {
+        if (a < 2) {
             un[a] = ui[a] + ph.dt * ((fi[a] + acc[a]) * im + ph.g[a]);
             xn[a] = xi[a] + ph.dt * un[a];
             // back into [0, n) on a periodic axis (a sub-step moves far less than a period)
@@ -635,10 +637,10 @@ __global__ void k_dem_substep(DemGeom g, DemPhys ph, DemBufs b, int early) {
             un[a] = ui[a];
             xn[a] = xi[a];
         }
-        const bool spin = (dim == 3) || (a == 2);
+        const bool spin = a == 2;
         on[a] = spin ? oi[a] + ph.dt * (ti[a] + acc[3 + a]) * iI : oi[a];
     }
-    const float disp2 = moved2(xn, xr, g.n, g.periodic, dim);
+    const float disp2 = moved2(xn, xr, g.n, g.periodic, 2);
     if (disp2 > 0.25f * (float)(g.skin * g.skin)) atomicAdd(&b.flags[3], 1);
     // a quarter of the skin used: the next call rebuilds the list
     if (disp2 > 0.0625f * (float)(g.skin * g.skin)) b.state[kRebuildReq] = 1;
@@ -647,6 +649,244 @@ __global__ void k_dem_substep(DemGeom g, DemPhys ph, DemBufs b, int early) {
     b.Xfo[i] = make_float4((float)xn[0], (float)xn[1], (float)xn[2], (float)ri);
     b.Vfo[2 * i] = make_float4((float)un[0], (float)un[1], (float)un[2], (float)on[0]);
     b.Vfo[2 * i + 1] = make_float4((float)on[1], (float)on[2], 0.0f, 0.0f);
+}
+
+constexpr int kSubThreads = 64;
+constexpr int kDemWide = 48;      // spheres per SM up to which eight lanes share one
+
+// One DEM sub-step of spheres. G lanes share a particle: a lane takes one neighbour slot (or, after
+// the slots, one near wall) at a time, so that a pass evaluates G contacts side by side. Their
+// forces and torques go through shared memory to the lane of each of the six components, which
+// adds them in FP64 (even and odd slots in rising order, then the walls, then the two sums: an order
+// that does not depend on G) and integrates that component.
+//
+// Bound by latency while few particles leave the chip idle (a contact is a chain of some 700
+// instructions, 15 cycles apart), by the FP64 pipe (1/64 of the FP32 rate: 50 % busy) beside it where
+// many do. So few particles take 8 lanes, one pass of contacts, and many take 2, with fewer FP64
+// instructions each. Ten sub-steps of a bed of touching spheres on a wall, two lanes walking the
+// slots one after the other before (one lane integrating; conversions on the FP64 pipe) / 2 / 8 lanes
+// now: 1536 spheres 195 / 187 / 111 us, 6144 200 / 192 / 142, 9216 197 / 191 / 232, 24576 287 / 259 /
+// 412, 49152 500 / 452 / 690; hence kDemWide per SM (7296 on 152 SMs). 4 lanes lie between: 153, 161,
+// 197, 349, 612. Smaller register budgets for more warps (80, 96) spill and gain nothing.
+// early = 1 when the kernel before it in the stream is the previous sub-step of the same call.
+template <int G>
+__global__ void __launch_bounds__(kSubThreads, 6) k_dem_substep3(DemGeom g, DemPhys ph, DemBufs b, int early) {
+    constexpr int NC = (6 + G - 1) / G;
+    __shared__ float s_ft[6][kSubThreads];
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = t / G, sub = t % G, lane = threadIdx.x & 31, first = lane - sub;
+    const bool valid = i < b.n;
+    // the k-th component (F and U along x, y, z, then T and Omega) of this lane, and its axis
+    auto comp = [&](const int k) { return sub + k * G; };
+    auto own = [&](const int k) { return valid && comp(k) < 6; };
+    auto lin = [&](const int k) { return comp(k) < 3; };
+    auto axis = [&](const int k) { return comp(k) < 3 ? comp(k) : comp(k) - 3; };
+    // Values fixed over a call's sub-steps: the list in use, the particle's neighbour count, the
+    // lane's first neighbour with its radius and mass, the particle's, the fluid's F or T and
+    // the position at the list's build. After a sub-step of the same call they are loaded before
+    // waiting for it, so the wait leads straight to the loads of the state that sub-step wrote.
+    int li = 0, nn = 0, j = 0;
+    double ri = 1.0, rj = 0.0, hyd[NC] = {}, xr[NC] = {}, im[NC] = {};
+    float imi = 0.0f, imj = 0.0f;
+    auto fixed = [&]() {
+        li = b.state[kListIdx];
+        if (!valid) return;
+        nn = (int)PSC_IDX(b.nbr_n[li][i], kNB + 1, CHK_NBR);
+        if (sub < nn) {
+            j = (int)PSC_IDX(b.nbr[li][i * kNB + sub], b.n, CHK_PART);
+            rj = b.R[j];
+            imj = to_f32(b.minv[2 * j]);
+        }
+        ri = b.R[i];
+        imi = to_f32(b.minv[2 * i]);
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            if (!own(k)) continue;
+            hyd[k] = (lin(k) ? b.Ff : b.Tf)[3 * i + axis(k)];
+            im[k] = b.minv[2 * i + (lin(k) ? 0 : 1)];
+            if (lin(k)) xr[k] = b.Xref[3 * i + axis(k)];
+        }
+    };
+    if (early) {
+        fixed();
+        dep_wait();
+    } else {
+        dep_wait();
+        fixed();
+    }
+    dep_launch();
+    const int *const nbr = b.nbr[li];
+    float *const hist = b.hist[li];
+    double xi[3] = {0, 0, 0}, x[NC] = {}, v[NC] = {}, acc[NC][2] = {};
+    float4 pif = make_float4(0.0f, 0.0f, 0.0f, 0.0f), vi0 = pif, vi1 = pif;
+    if (valid) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) xi[a] = b.X[3 * i + a];
+        pif = b.Xf[i];
+        vi0 = b.Vf[2 * i]; vi1 = b.Vf[2 * i + 1];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) {
+            if (!own(k)) continue;
+            v[k] = (lin(k) ? b.U : b.Om)[3 * i + axis(k)];
+            if (lin(k)) x[k] = b.X[3 * i + axis(k)];
+        }
+    }
+    const float uif[3] = {vi0.x, vi0.y, vi0.z};
+    const float oif[3] = {vi0.w, vi1.x, vi1.y};
+    int fail = 0;
+    // the axes on which a wall is near. Elsewhere there is no contact now, and there was none in
+    // the previous sub-step either (the skin exceeds the largest pull-off separation and a call's
+    // displacement), so that history is zero -- written, not read.
+    unsigned near = 0u;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (g.periodic[a] || !valid) continue;
+        const float xa = a == 0 ? pif.x : (a == 1 ? pif.y : pif.z);
+        const float dist = fminf(xa + 0.5f, ((float)g.n[a] - 0.5f) - xa);
+        if (pif.w - dist >= -(2.0f * (float)g.skin + g.margin)) {
+            near |= 1u << a;
+        } else if (sub == a % G) {
+            float4 *wp4 = reinterpret_cast<float4 *>(b.whist + ((size_t)i * 3 + a) * kH);
+            wp4[0] = wp4[1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+    }
+    const int items = valid ? nn + __popc(near) : 0;
+    const int passes = (__reduce_max_sync(kFullMask, items) + G - 1) / G;
+#pragma unroll 1
+    for (int p = 0; p < passes; ++p) {
+        const int s = p * G + sub;
+        bool contact = false, was = false, odd = s & 1;
+        float nv[3] = {0.0f, 0.0f, 0.0f}, ujf[3] = {0.0f, 0.0f, 0.0f}, ojf[3] = {0.0f, 0.0f, 0.0f};
+        float dnf = 0.0f, rjf = 0.0f, Rij = 1.0f;
+        float4 h0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), h1 = h0;
+        float4 *hp4 = nullptr;
+        if (s < nn && valid) {
+            if (p > 0) {
+                j = (int)PSC_IDX(nbr[i * kNB + s], b.n, CHK_PART);
+                rj = b.R[j];
+                imj = to_f32(b.minv[2 * j]);
+            }
+            hp4 = reinterpret_cast<float4 *>(hist + ((size_t)i * kNB + s) * kH);
+            // everything the pair may need, loaded at once
+            const float4 pj = b.Xf[j];
+            double xj[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+            for (int a = 0; a < 3; ++a) xj[a] = b.X[3 * j + a];
+            const float4 vj0 = b.Vf[2 * j], vj1 = b.Vf[2 * j + 1];
+            h0 = hp4[0]; h1 = hp4[1];
+            was = h1.w != 0.0f;
+            contact = pair_contact<3>(g, ph, b.reject, pif, pj, xi, xj, ri, rj, was, nv, dnf, Rij);
+            rjf = pj.w;
+            ujf[0] = vj0.x; ujf[1] = vj0.y; ujf[2] = vj0.z;
+            ojf[0] = vj0.w; ojf[1] = vj1.x; ojf[2] = vj1.y;
+        } else if (s < items) {
+            // contacts with the walls of the non-periodic axes (the fluid's halfway bounce-back
+            // planes at -1/2 and n - 1/2): the nearer wall is a half-space of the same material
+            // at rest (R = r_i, m* = m_i). The overlap and the decision are formed in FP64 with
+            // IEEE-rounded operations, as for the pairs.
+            unsigned m = near;
+            for (int w = s - nn; w > 0; --w) m &= m - 1u;
+            const int a = __ffs(m) - 1;
+            odd = a & 1;
+            auto of = [&](const double *v) { return a == 0 ? v[0] : (a == 1 ? v[1] : v[2]); };
+            const double xa = of(xi);
+            const bool lower = xa < of(g.mid);
+            const double dist = lower ? __dadd_rn(xa, 0.5) : __dsub_rn(of(g.hi_wall), xa);
+            const double dn = __dsub_rn(ri, dist);
+            hp4 = reinterpret_cast<float4 *>(b.whist + ((size_t)i * 3 + a) * kH);
+            {
+                h0 = hp4[0]; h1 = hp4[1];
+                was = h1.w != 0.0f;
+                if (!ph.adhesive) {
+                    contact = dn > 0.0;
+                } else if (dn >= 0.0) {
+                    contact = true;
+                } else if (was) {
+                    const double a064 = cbrt(9.0 * kPi * (double)ph.gamma * ri * ri / (double)ph.Es);
+                    contact = dn > -(a064 * a064 * ph.dc_coef / ri);
+                }
+                nv[0] = a == 0 ? (lower ? -1.0f : 1.0f) : 0.0f;
+                nv[1] = a == 1 ? (lower ? -1.0f : 1.0f) : 0.0f;
+                nv[2] = a == 2 ? (lower ? -1.0f : 1.0f) : 0.0f;
+                dnf = to_f32(dn);
+                Rij = to_f32(ri);
+                imj = 0.0f;
+            }
+        }
+        if (contact || was) {
+            float hl[kH] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+            float fo[3], to[3];
+            contact = contact_on_i(ph, 3, contact, nv, dnf, pif.w, rjf, Rij, 1.0f / (imi + imj), uif, ujf, oif, ojf, hl,
+                                   fo, to, &fail);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                s_ft[a][threadIdx.x] = fo[a];
+                s_ft[3 + a][threadIdx.x] = to[a];
+            }
+            hp4[0] = make_float4(hl[0], hl[1], hl[2], hl[3]);
+            hp4[1] = make_float4(hl[4], hl[5], hl[6], hl[7]);
+        }
+        // the contacts of the pass, added in slot order by the lane of each component
+        if (!__any_sync(kFullMask, contact)) continue;
+        const unsigned group = G == 32 ? kFullMask : ((1u << (G & 31)) - 1u) << first;
+        unsigned m0 = __ballot_sync(kFullMask, contact && !odd) & group;      // orders the stores above, too
+        unsigned m1 = __ballot_sync(kFullMask, contact && odd) & group;
+        __syncwarp();
+        if (valid) {
+            const float *const row = s_ft[0] + (threadIdx.x - lane);
+            while (m0 | m1) {
+                const int s0 = m0 ? __ffs(m0) - 1 : -1, s1 = m1 ? __ffs(m1) - 1 : -1;
+#pragma unroll
+                for (int k = 0; k < NC; ++k) {
+                    if (comp(k) >= 6) continue;
+                    if (s0 >= 0) acc[k][0] += to_f64(row[comp(k) * kSubThreads + s0]);
+                    if (s1 >= 0) acc[k][1] += to_f64(row[comp(k) * kSubThreads + s1]);
+                }
+                m0 &= m0 - 1u;
+                m1 &= m1 - 1u;
+            }
+        }
+        __syncwarp();
+    }
+    if (fail) atomicAdd(&b.flags[1], 1);
+    // Eq. 21, semi-implicit Euler, hydrodynamic force/torque frozen over the sub-steps:
+    // U + dt ((F + f) / m + g), Omega + dt (T + t) / I
+    float moved[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int k = 0; k < NC; ++k) {
+        const int a = axis(k);
+        auto along = [&](const auto p, const auto q, const auto r) { return a == 0 ? p : (a == 1 ? q : r); };
+        if (!own(k)) continue;
+        const double f = hyd[k] + (acc[k][0] + acc[k][1]);
+        const double q = __fma_rn(f, lin(k) ? im[k] : ph.dt, lin(k) ? along(ph.g[0], ph.g[1], ph.g[2]) : -0.0);
+        const double vn = __fma_rn(q, lin(k) ? ph.dt : im[k], v[k]);
+        (lin(k) ? b.Uo : b.Omo)[3 * i + a] = vn;
+        reinterpret_cast<float *>(b.Vfo + 2 * i)[comp(k)] = to_f32(vn);
+        if (lin(k)) {
+            double xn = __fma_rn(ph.dt, vn, x[k]);
+            // back into [0, n) on a periodic axis (a sub-step moves far less than a period)
+            const int per = along(g.periodic[0], g.periodic[1], g.periodic[2]);
+            if (per) {
+                const double len = along(g.len[0], g.len[1], g.len[2]);
+                const long long bits = __double_as_longlong(xn);      // ordered as numbers >= 0 are
+                if (bits < 0) { if (xn != 0.0) xn += len; }
+                else if (bits >= __double_as_longlong(len)) xn -= len;
+            }
+            const float mv = axis_moved(xn, xr[k], along(g.n[0], g.n[1], g.n[2]), per);
+            b.Xo[3 * i + a] = xn;
+            reinterpret_cast<float *>(b.Xfo + i)[a] = to_f32(xn);
+            if (a == sub) moved[0] = mv;                  // the lane's first axis,
+            else moved[2] = mv;                           // and of two lanes also the third
+        }
+    }
+    moved[1] = __shfl_down_sync(kFullMask, moved[0], 1);
+    if (G > 2) moved[2] = __shfl_down_sync(kFullMask, moved[0], 2);
+    if (!valid || sub != 0) return;
+    reinterpret_cast<float *>(b.Xfo + i)[3] = to_f32(ri);
+    const float disp2 = moved[0] * moved[0] + moved[1] * moved[1] + moved[2] * moved[2];
+    if (disp2 > 0.25f * (float)(g.skin * g.skin)) atomicAdd(&b.flags[3], 1);
+    // a quarter of the skin used: the next call rebuilds the list
+    if (disp2 > 0.0625f * (float)(g.skin * g.skin)) b.state[kRebuildReq] = 1;
 }
 
 }  // namespace
@@ -814,6 +1054,9 @@ extern "C" lbm_status dem_create(const dem_params *p, lbm_ctx *fluid, dem_ctx **
         d->g.n[a] = fluid->g.n[a];
         d->g.periodic[a] = fluid->g.periodic[a];
         d->g.inv_n[a] = 1.0 / fluid->g.n[a];
+        d->g.len[a] = fluid->g.n[a];
+        d->g.mid[a] = 0.5 * (fluid->g.n[a] - 1);
+        d->g.hi_wall[a] = fluid->g.n[a] - 0.5;
     }
     d->g.skin = p->skin > 0 ? p->skin : 0.5;
     d->ph.Es = (float)(p->E / (2.0 * (1.0 - p->poisson * p->poisson)));
@@ -898,16 +1141,20 @@ cudaError_t dem_enqueue_substeps(dem_ctx *d, int substeps, cudaStream_t s) {
     b.minv = d->minv;
     b.flags = fl->flags;
     b.reject = d->reject;
-    const int threads = 128;
-    const int blocks = (int)(((long long)n * kLPP + threads - 1) / threads);
+    int dev = 0, sms = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const bool wide = d->g.dim == 3 && n <= kDemWide * sms;
+    auto kern = d->g.dim == 2 ? k_dem_substep2 : (wide ? k_dem_substep3<8> : k_dem_substep3<2>);
+    const unsigned threads = d->g.dim == 2 ? 128u : (unsigned)kSubThreads;
+    const unsigned blocks = (unsigned)(((long long)n * (wide ? 8 : 2) + threads - 1) / threads);
     double *X[2] = {fl->dX, d->X2}, *U[2] = {fl->dU, d->U2}, *Om[2] = {fl->dOm, d->Om2};
     for (int k = 0; k < substeps && e == cudaSuccess; ++k) {
         const int src = k & 1, dst = src ^ 1;
         b.X = X[src]; b.U = U[src]; b.Om = Om[src]; b.Xf = d->Xf[src]; b.Vf = d->Vf[src];
         b.Xo = X[dst]; b.Uo = U[dst]; b.Omo = Om[dst]; b.Xfo = d->Xf[dst]; b.Vfo = d->Vf[dst];
         const int early = k > 0 ? 1 : 0;
-        if (d->g.dim == 2) e = launch_dep(k_dem_substep<2>, (unsigned)blocks, (unsigned)threads, s, d->g, d->ph, b, early);
-        else e = launch_dep(k_dem_substep<3>, (unsigned)blocks, (unsigned)threads, s, d->g, d->ph, b, early);
+        e = launch_dep(kern, blocks, threads, s, d->g, d->ph, b, early);
     }
     if (e != cudaSuccess) return e;
     return cudaGetLastError();

@@ -4,6 +4,7 @@
 #pragma once
 
 #include <math.h>
+#include <string.h>
 
 namespace psc {
 
@@ -92,22 +93,68 @@ __host__ __device__ __forceinline__ int axis_at(int k, int start, int nb, int pe
     return periodic ? (start + k) % nb : start + k;
 }
 
+// (float)v, rounded to nearest, and (double)v by integer operations for results that are normal
+// numbers: conversions run on the FP64 pipe, at 1/64 of the rate of these.
+__host__ __device__ __forceinline__ float to_f32(const double v) {
+#ifdef __CUDA_ARCH__
+    const unsigned long long w = (unsigned long long)__double_as_longlong(v);
+#else
+    unsigned long long w;
+    memcpy(&w, &v, sizeof(w));
+#endif
+    const unsigned hi = (unsigned)(w >> 32), lo = (unsigned)w, a = (hi & 0x7fffffffu) - 0x38000000u;
+    if (a - 0x00100000u >= 0x0fd00000u) return (float)v;       // below 2^-126, above 2^127, not a number
+    unsigned r = (a << 3) | (lo >> 29);
+    r += ((lo & 0x1fffffffu) + 0x0fffffffu + (r & 1u)) >> 29;      // half to even
+    r |= hi & 0x80000000u;
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(r);
+#else
+    float f;
+    memcpy(&f, &r, sizeof(f));
+    return f;
+#endif
+}
+__host__ __device__ __forceinline__ double to_f64(const float v) {
+#ifdef __CUDA_ARCH__
+    const unsigned b = __float_as_uint(v);
+#else
+    unsigned b;
+    memcpy(&b, &v, sizeof(b));
+#endif
+    const unsigned a = b & 0x7fffffffu;
+    if (a - 0x00800000u >= 0x7f000000u) return (double)v;      // zero, subnormal, not finite
+    const unsigned hi = (b & 0x80000000u) | ((a >> 3) + 0x38000000u), lo = a << 29;
+#ifdef __CUDA_ARCH__
+    return __hiloint2double((int)hi, (int)lo);
+#else
+    const unsigned long long w = ((unsigned long long)hi << 32) | lo;
+    double d;
+    memcpy(&d, &w, sizeof(d));
+    return d;
+#endif
+}
+
 // Squared displacement (FP32) of a particle at x from its position xr at the last
 // neighbour-list build: one image shift on a periodic axis, so the result is never below the
 // minimum-image displacement. The DEM rebuilds its list once a particle passes a quarter of
 // the skin; both the sub-step and a particle upload test this value.
+__host__ __device__ __forceinline__ float axis_moved(double x, double xr, int n, int periodic) {
+    float dd = to_f32(x - xr);
+    if (periodic) {
+        const float half = 0.5f * (float)n;
+        if (dd > half) dd -= (float)n;
+        else if (dd < -half) dd += (float)n;
+    }
+    return dd;
+}
 __host__ __device__ __forceinline__ float moved2(const double *x, const double *xr, const int *n, const int *periodic,
                                                  int dim) {
     float d2 = 0.0f;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         if (a >= dim) break;
-        float dd = (float)(x[a] - xr[a]);
-        if (periodic[a]) {
-            const float half = 0.5f * (float)n[a];
-            if (dd > half) dd -= (float)n[a];
-            else if (dd < -half) dd += (float)n[a];
-        }
+        const float dd = axis_moved(x[a], xr[a], n[a], periodic[a]);
         d2 += dd * dd;
     }
     return d2;
@@ -172,7 +219,7 @@ struct ContactSign {
 __host__ __device__ __forceinline__ ContactSign contact_sign(double d2, double S) {
     ContactSign c;
     const double u = dfma_rn(-S, S, d2);
-    const float d2f = (float)d2, uf = (float)u, Sf = (float)S;
+    const float d2f = to_f32(d2), uf = to_f32(u), Sf = to_f32(S);
     c.inv = rsqrt_f(d2f);
     c.ge0 = uf < 0.0f;
     c.gt0 = c.ge0;

@@ -53,6 +53,9 @@ extern "C" void psc_test_radii_range(const double *R, int n, double *s2min, doub
     radii_range(R, n, s2min, rmax);
 }
 
+extern "C" float psc_test_to_f32(double v) { return to_f32(v); }
+extern "C" double psc_test_to_f64(float v) { return to_f64(v); }
+
 extern "C" float psc_test_moved2(const double *x, const double *xr, const int *n, const int *periodic, int dim) {
     return moved2(x, xr, n, periodic, dim);
 }

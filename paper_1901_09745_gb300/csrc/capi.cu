@@ -552,8 +552,7 @@ extern "C" lbm_status lbm_set_particles(lbm_ctx *ctx, int n, const double *X, co
 // Queue the binning of the particles into the tiles' candidate lists (no host state).
 static lbm_status ctx_enqueue_bin(lbm_ctx *ctx) {
     Tiles tl = ctx_tiles(ctx);
-    CK(cudaMemsetAsync(ctx->tile_count, 0, (size_t)ctx->ntiles * sizeof(int), ctx->stream), "memset tile counts");
-    CK(cudaMemsetAsync(ctx->tile_stats, 0, kTileStats * sizeof(int), ctx->stream), "memset tile stats");
+    CK(launch_clear(ctx->tile_count, ctx->ntiles, ctx->tile_stats, NULL, NULL, 0, ctx->stream), "clear tile counts");
     CK(launch_bin(ctx->dim, ctx->g, ctx->ph, tl, ctx_parts(ctx), ctx->stream), "bin kernel");
     CK(launch_pack(ctx->q, ctx->p.storage, ctx->g, tl, ctx_parts(ctx), ctx->ntiles, ctx->stream), "pack kernel");
     return LBM_OK;
@@ -567,9 +566,7 @@ static lbm_status ctx_enqueue_step(lbm_ctx *ctx, bool bin, cudaEvent_t *ev) {
             lbm_status st = ctx_enqueue_bin(ctx);
             if (st != LBM_OK) return st;
         } else {
-            size_t v = (size_t)ctx->np * 3 * sizeof(double);
-            CK(cudaMemsetAsync(ctx->dF, 0, v, ctx->stream), "memset F");
-            CK(cudaMemsetAsync(ctx->dT, 0, v, ctx->stream), "memset T");
+            CK(launch_clear(NULL, 0, NULL, ctx->dF, ctx->dT, 3LL * ctx->np, ctx->stream), "clear F and T");
         }
     }
     if (ev) CK(cudaEventRecord(ev[0], ctx->stream), "cudaEventRecord");

@@ -173,6 +173,8 @@ cudaError_t launch_gather(int storage, int lattice, const void *fin, double *f_o
 cudaError_t launch_set(int storage, int lattice, const double *f, void *fout,
                        const Geom &g, const Phys &ph, cudaStream_t s);
 // Bin particles into tile candidate lists and zero F, T.
+// Clear ntiles counts (and stats unless null) and m values of F and T each.
+cudaError_t launch_clear(int *count, long long ntiles, int *stats, double *F, double *T, long long m, cudaStream_t s);
 cudaError_t launch_bin(int dim, const Geom &g, const Phys &ph, const Tiles &tl,
                        const Parts &pd, cudaStream_t s);
 // Sort each tile's list and write its packed candidate records (in the storage's compute type).

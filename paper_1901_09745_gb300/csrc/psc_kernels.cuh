@@ -877,8 +877,9 @@ __device__ __forceinline__ void psc_tile(const unsigned tile, const S *__restric
 #include "psc_pair16.cuh"
 
 // Tiles with more candidates than the block holds (rare): the exact chunked path over all
-// particles, one block per tile of the overflow list. With no such tile every block returns
-// at once.
+// particles, one block per tile of the overflow list. Its tiles are no other kernel's, so after
+// k_step (which starts it early, see launch_step_t; by then the lists are there) it works beside it
+// and only ends after it. With no such tile its launch then costs what its end does.
 template <class L, typename S, int PSC>
 __global__ void __launch_bounds__(kThreads, 1)
 k_collide_overflow(const S *__restrict__ fin, S *__restrict__ fout, Geom g, PhysT<typename Store<S>::T> ph,
@@ -888,14 +889,16 @@ k_collide_overflow(const S *__restrict__ fin, S *__restrict__ fout, Geom g, Phys
     __shared__ unsigned long long s_mask[kWarps];
     const long long ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
     const int novf = tl.stats[2];
-    // the 16-bit kernel before this one has finished: clear its work counters
-    if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) {
-        tl.stats[3] = 0;
-        tl.stats[6] = 0;
-    }
+    pdl_launch();
     for (int it = blockIdx.x; it < novf; it += gridDim.x) {
         psc_tile<L, S, PSC>(tl.order[2 * ntiles + it], fin, fout, g, ph, tl, pd, flags, reinterpret_cast<T *>(smem), s_mask);
         __syncthreads();
+    }
+    pdl_wait();
+    // the 16-bit kernel before this one has finished: clear its work counters
+    if (sizeof(S) == 2 && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) {
+        tl.stats[3] = 0;
+        tl.stats[6] = 0;
     }
 }
 
@@ -1143,13 +1146,17 @@ cudaError_t launch_overflow(const void *fin, void *fout, const Geom &g, const Ph
         cudaError_t e = cudaFuncSetAttribute(okern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osmem);
         if (e != cudaSuccess) return e;
     }
-    okern<<<32, dim3(L::TX, L::TY, L::TZ), osmem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
+    const dim3 block(L::TX, L::TY, L::TZ);
+    if (sizeof(S) != 2) return launch_pdl(okern, dim3(32), block, osmem, s, (const S *)fin, (S *)fout, g, pt, tl, pd, flags);
+    okern<<<32, block, osmem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
     return cudaGetLastError();
 }
 
 // Fluid-tile blocks per SM when they follow the particle tiles beside the caller's next
-// kernels (a deferred join).
-constexpr int kDeferF = 2;
+// kernels (a deferred join). 20 coupled steps of 2048^2 with 5000 discs, 5 of 4096^2 with 20000,
+// ms: 2 blocks 2.98 and 2.84, 3 2.93 and 2.63, 4 2.98 and 2.58, 5 3.17 and 2.73 (the
+// caller's kernels find no room beside them).
+constexpr int kDeferF = 3;
 
 // One launch of the step's kernel over the tiles of kind `which` (blocks_per_sm > 0 limits it).
 template <class L, typename S, int PSC, bool SOLID, bool VEC>
@@ -1171,7 +1178,10 @@ cudaError_t launch_step_t(const void *fin, void *fout, const Geom &g, const Phys
     e = persistent_blocks(kern, 0, (items + threads / 32 - 1) / (threads / 32), nb, threads);
     if (e != cudaSuccess) return e;
     if (blocks_per_sm > 0 && nb > (unsigned)(blocks_per_sm * sms)) nb = (unsigned)(blocks_per_sm * sms);
-    kern<<<nb, threads, 0, s>>>(Dirs<L, S>(fin, fout, g), g, pt, tl, pd, flags, tl.work, which, shift);
+    const Dirs<L, S> f(fin, fout, g);
+    if (which != kFluidTiles)      // (on the second stream after an event: the usual order)
+        return launch_pdl(kern, dim3(nb), dim3((unsigned)threads), 0, s, f, g, pt, tl, pd, flags, tl.work, which, shift);
+    kern<<<nb, threads, 0, s>>>(f, g, pt, tl, pd, flags, tl.work, which, shift);
     return cudaGetLastError();
 }
 
@@ -1223,7 +1233,7 @@ cudaError_t launch_collide_stream16(const void *fin, void *fout, const Geom &g, 
     using T = typename Store<S>::T;
     constexpr bool kSteal = L::D == 3;
     // blocks per SM side by side (2D): 4 x 128 threads x 80 registers + 3 x 128 x 64 = 64 K
-    constexpr int kSideP = 4, kSideF = 3;
+    constexpr int kSideP = 4, kSideF = 3, kDeferF16 = 2;
     const size_t smem = h16::pair_smem_bytes<L, T>();
     auto kern = h16::k_collide_stream<L, S, PSC, kSteal>;
     if (smem > 48 * 1024) {
@@ -1263,7 +1273,7 @@ cudaError_t launch_collide_stream16(const void *fin, void *fout, const Geom &g, 
         if (e == cudaSuccess) e = cudaEventRecord(ov->fork, s);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(ov->aux, ov->fork, 0);
         if (e != cudaSuccess) return e;
-        fkern<<<nsm * kDeferF, pblock, 0, ov->aux>>>(f, g, pt, tl, pd.n, flags);
+        fkern<<<nsm * kDeferF16, pblock, 0, ov->aux>>>(f, g, pt, tl, pd.n, flags);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaEventRecord(ov->join, ov->aux);
         if (e == cudaSuccess) ov->deferred = 1;

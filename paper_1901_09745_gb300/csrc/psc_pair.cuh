@@ -597,6 +597,8 @@ k_step(const __grid_constant__ Dirs<L, S> f, const __grid_constant__ Geom g,
     using T = typename Store<S>::T;
     using V = typename Pr<T>::V;
     __shared__ V s_slots[SOLID ? kPWarps * kSlots * 32 : 1];
+    pdl_wait();
+    pdl_launch();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned ntiles = (unsigned)g.nt[0] * (unsigned)g.nt[1] * (unsigned)g.nt[2];
     const unsigned np = (SOLID && (which & kParticleTiles)) ? (unsigned)tl.stats[4] : 0u;

@@ -33,8 +33,10 @@ namespace psc {
 
 template <class L, typename T>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 4 : 2)
-k_adjoint(const T *__restrict__ gt, const T *__restrict__ lam_in, T *__restrict__ lam_out, Geom g,
-          PhysT<T> ph, Tiles tl, Parts pd, T invT, double *dJdX, double *dFpart) {
+k_adjoint(const __grid_constant__ Dirs<L, T> fwd, const __grid_constant__ Dirs<L, T> adj, const __grid_constant__ Geom g,
+          const __grid_constant__ PhysT<T> ph, Tiles tl, Parts pd, T invT, double *dJdX, double *dFpart) {
+    const T *const gt = fwd.in[0];
+    T *const lam_out = const_cast<T *>(adj.in[0]);
     constexpr int Q = L::Q;
     constexpr int D = L::D;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -60,9 +62,13 @@ k_adjoint(const T *__restrict__ gt, const T *__restrict__ lam_in, T *__restrict_
     // address their neighbours by a fixed offset (no wrap or wall tests)
     const bool interior = x0 >= 1 && x0 + L::TX < g.n[0] && y0 >= 1 && y0 + L::TY < g.n[1] &&
                           (L::D == 2 || (z0 >= 1 && z0 + L::TZ < g.n[2]));
-    const long long sy = g.n[0], sz = (long long)g.n[0] * g.n[1];
     T d[Q];
-    pull_q<L, T>(gt, g, x, y, z, cell, interior, active, ph.sc, d);
+    if (interior) {
+#pragma unroll
+        for (int i = 0; i < Q; ++i) d[i] = *src_at<L, T>(fwd, g, i, cell - L::ex(i));
+    } else {
+        pull_q<L, T>(gt, g, x, y, z, cell, false, active, ph.sc, d);
+    }
     T drho = 0, j[3] = {0, 0, 0};
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -101,7 +107,7 @@ k_adjoint(const T *__restrict__ gt, const T *__restrict__ lam_in, T *__restrict_
     // two products lambda.d, lambda.d_opp, because f^eq and the Guo term are quadratic in e.
     T lam[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) lam[i] = active ? lam_in[(long long)i * N + cell] : (T)0;
+    for (int i = 0; i < Q; ++i) lam[i] = interior || active ? *dst_at<L, T>(adj, g, i, cell) : (T)0;
     T S0 = 0, S1[3] = {0, 0, 0}, Mxx = 0, Myy = 0, Mzz = 0, Mxy = 0, Mxz = 0, Myz = 0, Ld = 0, Ldo = 0;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -165,7 +171,7 @@ k_adjoint(const T *__restrict__ gt, const T *__restrict__ lam_in, T *__restrict_
             if (L::ey(k)) a += L::ey(k) > 0 ? Av[1] : -Av[1];
             if (L::ez(k)) a += L::ez(k) > 0 ? Av[2] : -Av[2];
             if (interior) {
-                lam_out[(long long)k * N + cell - (L::ex(k) + L::ey(k) * sy + L::ez(k) * sz)] = a;
+                *const_cast<T *>(src_at<L, T>(adj, g, k, cell - L::ex(k))) = a;
             } else {
                 lam_out[src_index<L>(nb, k, cell, N)] = a;   // S^T: the pull's source, written once
             }
@@ -278,7 +284,8 @@ cudaError_t launch_adjoint_t(const void *gt, const void *lam_in, void *lam_out, 
     }
     dim3 grid(g.nt[0], g.nt[1], g.nt[2]);
     dim3 block(L::TX, L::TY, L::TZ);
-    kern<<<grid, block, smem, s>>>((const T *)gt, (const T *)lam_in, (T *)lam_out, g, make_phys<T>(ph, L::Q), tl, pd,
+    kern<<<grid, block, smem, s>>>(Dirs<L, T>(gt, const_cast<void *>(gt), g),
+                                   Dirs<L, T>(lam_out, const_cast<void *>(lam_in), g), g, make_phys<T>(ph, L::Q), tl, pd,
                                    (T)invT, dJdX, dFpart);
     return cudaGetLastError();
 }

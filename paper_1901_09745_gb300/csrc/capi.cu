@@ -608,6 +608,14 @@ static lbm_status ctx_step_graph(lbm_ctx *ctx, bool bin, bool *done) {
     return LBM_OK;
 }
 
+// The kernels of one step: what it accumulates into cleared, then those of launch_collide_stream.
+static int ctx_step_kernels(const lbm_ctx *ctx, const bool deferred) {
+    if (ctx->np == 0) return 1;
+    if (open_faces(ctx->g)) return 3;
+    if (ctx->elem == 2) return ctx->dim == 2 ? 4 : 3;
+    return 2 + (deferred ? 1 : 0) + (may_overflow(ctx->p.tile_cap, ctx->np) ? 1 : 0);
+}
+
 lbm_status ctx_step_once(lbm_ctx *ctx) {
     const bool bin = ctx->np > 0 && !ctx->bins_valid;
     const bool timed = ctx->timing > 0 && ctx->steps % ctx->timing == 0;
@@ -638,8 +646,7 @@ lbm_status ctx_step_once(lbm_ctx *ctx) {
         ctx->launches += 2;
         ctx->bins_valid = 1;
     }
-    // the step's kernel (16 bits in 2D: two), the overflow tiles; open faces: two kernels
-    ctx->launches += (ctx->np > 0) ? ((ctx->dim == 2 && ctx->elem == 2 && !open_faces(ctx->g)) ? 3 : 2) : 1;
+    ctx->launches += ctx_step_kernels(ctx, false);
     ctx->cs_launches += 1;
     ctx->cur ^= 1;
     ctx->steps += 1;
@@ -718,7 +725,7 @@ static lbm_status ctx_coupled_once(lbm_ctx *ctx, dem_ctx *dem, int substeps) {
         ctx->launches += 2;
         ctx->bins_valid = 1;
     }
-    ctx->launches += open_faces(ctx->g) ? 2 : 3;
+    ctx->launches += ctx_step_kernels(ctx, true);
     ctx->cs_launches += 1;
     ctx->cur ^= 1;
     ctx->steps += 1;

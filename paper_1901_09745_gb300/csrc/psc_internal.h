@@ -173,6 +173,10 @@ cudaError_t launch_gather(int storage, int lattice, const void *fin, double *f_o
 cudaError_t launch_set(int storage, int lattice, const double *f, void *fout,
                        const Geom &g, const Phys &ph, cudaStream_t s);
 // Bin particles into tile candidate lists and zero F, T.
+// Candidates a tile may have in the step's usual kernels; tiles with more overflow, which takes more
+// particles (no particle is on a tile's list twice).
+constexpr int kPairCap = 32;
+__host__ inline bool may_overflow(const int cap, const int n) { return n > (cap < kPairCap ? cap : kPairCap); }
 // Clear ntiles counts (and stats unless null) and m values of F and T each.
 cudaError_t launch_clear(int *count, long long ntiles, int *stats, double *F, double *T, long long m, cudaStream_t s);
 cudaError_t launch_bin(int dim, const Geom &g, const Phys &ph, const Tiles &tl,

@@ -39,7 +39,6 @@ namespace psc {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kPairCap = 32;     // candidates a tile may have to take the two-cells-per-thread path
 
 template <typename T> struct PhysT {
     T omega;        // 1/tau
@@ -455,6 +454,19 @@ __global__ void k_pack_tiles(Geom g, Tiles tl, Parts pd, long long ntiles) {
     const bool valid = tx < g.nt[0];
     const int cnt = valid ? tl.count[tile] : -1;
     if (lane == 0) s_cnt[warp] = cnt;
+    __syncthreads();
+    // the lists first: their atomics are under way while the records are written
+    if (warp == 0) {
+        const int c = lane < kWarps ? s_cnt[lane] : -1, lim = min(tl.cap, kPairCap);
+        const unsigned mp = __ballot_sync(kFull, c > 0), mf = __ballot_sync(kFull, c == 0), mo = __ballot_sync(kFull, c > lim);
+        const unsigned mine = lane == 0 ? mp : (lane == 1 ? mf : (lane == 2 ? mo : 0u));
+        const int at = mine ? atomicAdd(&tl.stats[lane == 0 ? 4 : (lane == 1 ? 5 : 2)], __popc(mine)) : 0;
+        const int bp = __shfl_sync(kFull, at, 0), bf = __shfl_sync(kFull, at, 1), bo = __shfl_sync(kFull, at, 2);
+        const unsigned below = (1u << lane) - 1u, ent = (unsigned)(tile + lane);      // the first warp's tile + lane
+        if (c > 0) tl.order[bp + __popc(mp & below)] = ent;
+        else if (c == 0) tl.order[ntiles + bf + __popc(mf & below)] = ent;
+        if (c > lim) tl.order[2 * ntiles + bo + __popc(mo & below)] = ent;
+    }
     if (valid) {
         const int m = min(cnt, tl.cap);
         T *blk = reinterpret_cast<T *>(tl.blocks) + tile * block_elems<T>(tl.cap);
@@ -467,24 +479,6 @@ __global__ void k_pack_tiles(Geom g, Tiles tl, Parts pd, long long ntiles) {
             for (int q = 0; q < m; ++q) rank += (s_id[warp][q] < id);
             write_record<L, T>(blk + head_elems<T>() + (long long)rank * RW, g, pd, id, tx * L::TX, ty * L::TY,
                                tz * L::TZ);
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int np = 0, nf = 0;
-        for (int w = 0; w < kWarps; ++w) { np += (s_cnt[w] > 0); nf += (s_cnt[w] == 0); }
-        int no = 0;
-        const int lim = min(tl.cap, kPairCap);
-        for (int w = 0; w < kWarps; ++w) no += (s_cnt[w] > lim);
-        int bp = np ? atomicAdd(&tl.stats[4], np) : 0;
-        int bf = nf ? atomicAdd(&tl.stats[5], nf) : 0;
-        int bo = no ? atomicAdd(&tl.stats[2], no) : 0;
-        for (int w = 0; w < kWarps; ++w) {
-            if (s_cnt[w] < 0) continue;
-            const unsigned ent = (unsigned)(tile + w);      // thread 0's warp is the first
-            if (s_cnt[w] > 0) tl.order[bp++] = ent;
-            else tl.order[ntiles + bf++] = ent;
-            if (s_cnt[w] > lim) tl.order[2 * ntiles + bo++] = ent;
         }
     }
 }
@@ -1200,7 +1194,7 @@ cudaError_t launch_collide_stream_t(const void *fin, void *fout, const Geom &g, 
     const bool defer = ov && ov->aux && ov->defer && L::D == 2 && sizeof(T) == 4;
     cudaError_t e = launch_step_t<L, S, PSC, true, VEC>(fin, fout, g, pt, tl, pd, flags,
                                                               defer ? kParticleTiles : kBothLists, 0, s);
-    if (e == cudaSuccess) e = launch_overflow<L, S, PSC>(fin, fout, g, pt, tl, pd, flags, s);
+    if (e == cudaSuccess && may_overflow(tl.cap, pd.n)) e = launch_overflow<L, S, PSC>(fin, fout, g, pt, tl, pd, flags, s);
     if (e != cudaSuccess || !defer) return e;
     e = cudaEventRecord(ov->fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(ov->aux, ov->fork, 0);

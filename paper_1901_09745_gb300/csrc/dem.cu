@@ -463,6 +463,15 @@ __device__ __forceinline__ bool pair_contact(const DemGeom &g, const DemPhys &ph
     return dn > -(a064 * a064 * ph.dc_coef / R64);
 }
 
+// x back into [0, len) on a periodic axis (a sub-step moves far less than a period); the bits of
+// numbers >= 0 are ordered as they are, which spares the FP64 pipe two comparisons.
+__device__ __forceinline__ double wrapped(double x, const double len) {
+    const long long bits = __double_as_longlong(x);
+    if (bits < 0) { if (x != 0.0) x += len; }
+    else if (bits >= __double_as_longlong(len)) x -= len;
+    return x;
+}
+
 constexpr int kLPP = 2;   // lanes per particle in the sub-step kernel of discs (a coupled step of 5000:
                           // 1 lane 182.9 us, 2 lanes 162.0, 4 lanes 170.2, 8 lanes 206.0)
 
@@ -489,7 +498,7 @@ __global__ void k_dem_substep2(DemGeom g, DemPhys ph, DemBufs b, int early) {
         nn = (int)PSC_IDX(b.nbr_n[li][i], kNB + 1, CHK_NBR);
         jn = b.nbr[li][i * kNB + sub];      // the lane's first neighbour (read without waiting for nn)
         ri = b.R[i];
-        imi = (float)b.minv[2 * i];
+        imi = to_f32(b.minv[2 * i]);
         if (sub == 0) {
 #pragma unroll
             for (int a = 0; a < 3; ++a) { fi[a] = b.Ff[3 * i + a]; ti[a] = b.Tf[3 * i + a]; xr[a] = b.Xref[3 * i + a]; }
@@ -530,7 +539,7 @@ __global__ void k_dem_substep2(DemGeom g, DemPhys ph, DemBufs b, int early) {
             for (int a = 0; a < 3; ++a) if (a < 2) xj[a] = b.X[3 * j + a];
             const double rj = b.R[j];
             const float4 vj0 = b.Vf[2 * j], vj1 = b.Vf[2 * j + 1];
-            const float imj = (float)b.minv[2 * j];
+            const float imj = to_f32(b.minv[2 * j]);
             float4 *hp4 = reinterpret_cast<float4 *>(hp);
             const float4 h0 = hp4[0], h1 = hp4[1];
             const bool was = h1.w != 0.0f;
@@ -549,8 +558,8 @@ __global__ void k_dem_substep2(DemGeom g, DemPhys ph, DemBufs b, int early) {
                              &fail)) {
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
-                    if (used(a)) acc[a] += (double)fo[a];
-                    if (used(3 + a)) acc[3 + a] += (double)to[a];
+                    if (used(a)) acc[a] += to_f64(fo[a]);
+                    if (used(3 + a)) acc[3 + a] += to_f64(to[a]);
                 }
             }
             hp4[0] = make_float4(hl[0], hl[1], hl[2], hl[3]);
@@ -564,9 +573,8 @@ __global__ void k_dem_substep2(DemGeom g, DemPhys ph, DemBufs b, int early) {
 #pragma unroll
     for (int a = 0; a < 2; ++a) {       // unrolled: the per-axis arrays stay in registers
         if (!valid || a % kLPP != sub || g.periodic[a]) continue;
-        const double lo_plane = 0.5 * (double)(g.n[a] - 1);
-        const bool lower = xi[a] < lo_plane;
-        const double dist = lower ? __dadd_rn(xi[a], 0.5) : __dsub_rn((double)g.n[a] - 0.5, xi[a]);
+        const bool lower = xi[a] < g.mid[a];
+        const double dist = lower ? __dadd_rn(xi[a], 0.5) : __dsub_rn(g.hi_wall[a], xi[a]);
         const double dn = __dsub_rn(ri, dist);
         float4 *wp4 = reinterpret_cast<float4 *>(b.whist + ((size_t)i * 3 + a) * kH);
         if (dn < -2.0 * g.skin) {
@@ -605,8 +613,8 @@ __global__ void k_dem_substep2(DemGeom g, DemPhys ph, DemBufs b, int early) {
                              &fail)) {
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    if (used(c)) acc[c] += (double)fo[c];
-                    if (used(3 + c)) acc[3 + c] += (double)to[c];
+                    if (used(c)) acc[c] += to_f64(fo[c]);
+                    if (used(3 + c)) acc[3 + c] += to_f64(to[c]);
                 }
             }
             wp4[0] = make_float4(hl[0], hl[1], hl[2], hl[3]);
@@ -630,8 +638,7 @@ __global__ void k_dem_substep2(DemGeom g, DemPhys ph, DemBufs b, int early) {
             xn[a] = xi[a] + ph.dt * un[a];
             // back into [0, n) on a periodic axis (a sub-step moves far less than a period)
             if (g.periodic[a]) {
-                if (xn[a] < 0.0) xn[a] += (double)g.n[a];
-                else if (xn[a] >= (double)g.n[a]) xn[a] -= (double)g.n[a];
+                xn[a] = wrapped(xn[a], g.len[a]);
             }
         } else {
             un[a] = ui[a];
@@ -646,9 +653,9 @@ __global__ void k_dem_substep2(DemGeom g, DemPhys ph, DemBufs b, int early) {
     if (disp2 > 0.0625f * (float)(g.skin * g.skin)) b.state[kRebuildReq] = 1;
 #pragma unroll
     for (int a = 0; a < 3; ++a) { b.Xo[3 * i + a] = xn[a]; b.Uo[3 * i + a] = un[a]; b.Omo[3 * i + a] = on[a]; }
-    b.Xfo[i] = make_float4((float)xn[0], (float)xn[1], (float)xn[2], (float)ri);
-    b.Vfo[2 * i] = make_float4((float)un[0], (float)un[1], (float)un[2], (float)on[0]);
-    b.Vfo[2 * i + 1] = make_float4((float)on[1], (float)on[2], 0.0f, 0.0f);
+    b.Xfo[i] = make_float4(to_f32(xn[0]), to_f32(xn[1]), to_f32(xn[2]), to_f32(ri));
+    b.Vfo[2 * i] = make_float4(to_f32(un[0]), to_f32(un[1]), to_f32(un[2]), to_f32(on[0]));
+    b.Vfo[2 * i + 1] = make_float4(to_f32(on[1]), to_f32(on[2]), 0.0f, 0.0f);
 }
 
 constexpr int kSubThreads = 64;
@@ -866,12 +873,7 @@ __global__ void __launch_bounds__(kSubThreads, 6) k_dem_substep3(DemGeom g, DemP
             double xn = __fma_rn(ph.dt, vn, x[k]);
             // back into [0, n) on a periodic axis (a sub-step moves far less than a period)
             const int per = along(g.periodic[0], g.periodic[1], g.periodic[2]);
-            if (per) {
-                const double len = along(g.len[0], g.len[1], g.len[2]);
-                const long long bits = __double_as_longlong(xn);      // ordered as numbers >= 0 are
-                if (bits < 0) { if (xn != 0.0) xn += len; }
-                else if (bits >= __double_as_longlong(len)) xn -= len;
-            }
+            if (per) xn = wrapped(xn, along(g.len[0], g.len[1], g.len[2]));
             const float mv = axis_moved(xn, xr[k], along(g.n[0], g.n[1], g.n[2]), per);
             b.Xo[3 * i + a] = xn;
             reinterpret_cast<float *>(b.Xfo + i)[a] = to_f32(xn);

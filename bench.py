@@ -32,7 +32,7 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 FALLBACK_HBM_GBS = 6800.0
-KERNEL_FILES = ["psc_kernels.cuh", "psc_pair.cuh", "lattice.cuh", "psc_internal.h", "psc_f32.cu"]
+KERNEL_FILES = ["psc_kernels.cuh", "psc_pair.cuh", "psc_pair16.cuh", "lattice.cuh", "psc_internal.h", "psc_f32.cu"]
 
 
 def parse_args(argv=None):
@@ -352,7 +352,7 @@ def run_ours(args, rank, local_rank, world):
                    "l2": "inputs larger than L2: %.0f MB of populations read+written per step"
                          % (bytes_per_launch / 1e6),
                    "parallelism": "replicas (one independent domain per GPU)"},
-        "roofline": {"bound": "hbm", "kernel": "k_collide_stream with k_fluid_pair and k_collide_overflow "
+        "roofline": {"bound": "hbm", "kernel": "k_step with k_collide_overflow "
                                                "(one collide-stream step)", "achieved": round(achieved, 1),
                      "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4),
                      "peak_source": peak_kind, "traffic": traffic,

@@ -298,9 +298,7 @@ cudaError_t launch_adjoint(int storage, int lattice, const void *gt, const void 
                             : launch_adjoint_t<D3Q19, double>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
     }
     if (lattice == 9) return launch_adjoint_t<D2Q9, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
-    return g.wide
-               ? launch_adjoint_t<D3Q19w, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s)
-               : launch_adjoint_t<D3Q19, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
+    return launch_adjoint_t<D3Q19, float>(gt, lam_in, lam_out, g, ph, tl, pd, invT, dJdX, dFpart, s);
 }
 
 }  // namespace psc
@@ -349,6 +347,36 @@ static AdjSpace adj_layout(const lbm_ctx *ctx, int nsteps, int K) {
     return a;
 }
 
+// The adjoint's steps in FP32 keep the order of roundings they have by the pair kernels (see
+// launch_collide_stream_l), on narrow tiles, whose candidates decide what lbm_adjoint_forward
+// refuses: while this lives, the context's steps, lists and graphs are those.
+struct KeepOrder {
+    lbm_ctx *const ctx;
+    const Geom g;
+    const long long ntiles;
+    explicit KeepOrder(lbm_ctx *c) : ctx(c), g(c->g), ntiles(c->ntiles) {
+        if (ctx->p.storage != LBM_F32) return;
+        ctx->keep = 1;
+        if (!g.wide) return;
+        ctx->g.wide = 0;
+        for (int a = 0; a < 3; ++a) {
+            const int ext = tile_ext(ctx->dim, 0, a);
+            ctx->g.nt[a] = (g.n[a] + ext - 1) / ext;
+            const double need = ext + 2.0 * (ctx->rmax + ctx->p.shell_h) + 2.0;
+            ctx->g.wrap_img[a] = (a < ctx->dim && g.periodic[a] && g.n[a] < need) ? 1 : 0;
+        }
+        ctx->ntiles = tile_number(ctx->dim, 0, g);
+        ctx->bins_valid = 0;
+    }
+    ~KeepOrder() {
+        ctx->keep = 0;
+        if (!g.wide) return;
+        ctx->g = g;
+        ctx->ntiles = ntiles;
+        ctx->bins_valid = 0;
+    }
+};
+
 // Forward half: T steps from the context's state with a checkpoint every K, J summed on the
 // device. Leaves the checkpoints and the tile lists for lbm_adjoint_backward.
 extern "C" lbm_status lbm_adjoint_forward(lbm_ctx *ctx, int nsteps, int checkpoint_every, double *J,
@@ -366,6 +394,7 @@ extern "C" lbm_status lbm_adjoint_forward(lbm_ctx *ctx, int nsteps, int checkpoi
             ctx_error(ctx, "the adjoint supports periodic and wall axes only");
             return LBM_ERR_UNSUPPORTED;
         }
+    const KeepOrder keep(ctx);
     const int n = ctx->np;
     const int K = checkpoint_every;
     lbm_status status = LBM_OK;
@@ -450,6 +479,7 @@ extern "C" lbm_status lbm_adjoint_backward(lbm_ctx *ctx, long long token, double
         ctx_error(ctx, "the particles or the body force changed since lbm_adjoint_forward");
         return LBM_ERR_ARG;
     }
+    const KeepOrder keep(ctx);
     const int n = ctx->np;
     const int nsteps = ctx->adj_T, K = ctx->adj_K;
     lbm_status status = LBM_OK;
@@ -464,9 +494,15 @@ extern "C" lbm_status lbm_adjoint_backward(lbm_ctx *ctx, long long token, double
         tl.count = ctx->tile_count; tl.list = ctx->tile_list; tl.cap = ctx->p.tile_cap;
         tl.stats = ctx->tile_stats; tl.blocks = ctx->tile_blocks; tl.order = ctx->tile_order;
         tl.work = ctx->step_work;
+        tl.keep = ctx->keep;
         scratch_parts = ctx_parts(ctx);
         scratch_parts.F = w.sF;
         scratch_parts.T = w.sT;
+        if (n > 0 && !ctx->bins_valid) {
+            ACK(launch_clear(ctx->tile_count, ctx->ntiles, ctx->tile_stats, NULL, NULL, 0, ctx->stream), "clear tile counts");
+            ACK(launch_bin(ctx->dim, ctx->g, ctx->ph, tl, scratch_parts, ctx->stream), "bin kernel");
+            ACK(launch_pack(ctx->q, ctx->p.storage, ctx->g, tl, scratch_parts, ctx->ntiles, ctx->stream), "pack kernel");
+        }
         // segment by segment: restore the checkpoint, re-run the segment storing its states,
         // walk it back
         int cur = 0;

@@ -282,10 +282,10 @@ extern "C" lbm_status lbm_destroy(lbm_ctx *ctx) {
     free_dev(&ctx->adj);
     for (int i = 0; i < ctx->ev_cap; ++i) cudaEventDestroy(ctx->ev[i]);
     free(ctx->ev);
-    for (int a = 0; a < 2; ++a)
+    for (int a = 0; a < 4; ++a)
         for (int b = 0; b < 2; ++b) {
             if (ctx->sgraph[a][b]) cudaGraphExecDestroy(ctx->sgraph[a][b]);
-            if (ctx->cgraph[a][b]) cudaGraphExecDestroy(ctx->cgraph[a][b]);
+            if (a < 2 && ctx->cgraph[a][b]) cudaGraphExecDestroy(ctx->cgraph[a][b]);
         }
     if (ctx->ov.aux) cudaStreamDestroy(ctx->ov.aux);
     if (ctx->ov.fork) cudaEventDestroy(ctx->ov.fork);
@@ -310,6 +310,7 @@ static Tiles ctx_tiles(lbm_ctx *ctx) {
     tl.order = ctx->tile_order;
     tl.blocks = ctx->tile_blocks;
     tl.work = ctx->step_work;
+    tl.keep = ctx->keep;
     return tl;
 }
 
@@ -371,11 +372,13 @@ lbm_status ctx_reserve_particles(lbm_ctx *ctx, int n) {
 static lbm_status ctx_reserve_tiles(lbm_ctx *ctx) {
     if (ctx->tile_count) return LBM_OK;
     ctx->gen += 1;
-    CK(cudaMalloc(&ctx->tile_count, (size_t)ctx->ntiles * sizeof(int)), "cudaMalloc(tile counts)");
-    CK(cudaMalloc(&ctx->tile_list, (size_t)ctx->ntiles * ctx->p.tile_cap * sizeof(int)), "cudaMalloc(tile lists)");
+    // (the adjoint cuts the lattice into narrow tiles)
+    const long long narrow = tile_number(ctx->dim, 0, ctx->g), room = narrow > ctx->ntiles ? narrow : ctx->ntiles;
+    CK(cudaMalloc(&ctx->tile_count, (size_t)room * sizeof(int)), "cudaMalloc(tile counts)");
+    CK(cudaMalloc(&ctx->tile_list, (size_t)room * ctx->p.tile_cap * sizeof(int)), "cudaMalloc(tile lists)");
     CK(cudaMalloc(&ctx->tile_stats, kTileStats * sizeof(int)), "cudaMalloc(tile stats)");
-    CK(cudaMalloc(&ctx->tile_order, (size_t)ctx->ntiles * 3 * sizeof(unsigned)), "cudaMalloc(tile order)");
-    CK(cudaMalloc(&ctx->tile_blocks, (size_t)ctx->ntiles * pack_block_bytes(ctx->p.storage == LBM_F64, ctx->p.tile_cap)),
+    CK(cudaMalloc(&ctx->tile_order, (size_t)room * 3 * sizeof(unsigned)), "cudaMalloc(tile order)");
+    CK(cudaMalloc(&ctx->tile_blocks, (size_t)room * pack_block_bytes(ctx->p.storage == LBM_F64, ctx->p.tile_cap)),
        "cudaMalloc(tile candidate blocks)");
     CK(cudaMemsetAsync(ctx->tile_stats, 0, kTileStats * sizeof(int), ctx->stream), "memset tile stats");
     return LBM_OK;
@@ -585,9 +588,11 @@ static lbm_status ctx_step_graph(lbm_ctx *ctx, bool bin, bool *done) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     CK(cudaStreamIsCapturing(ctx->stream, &cs), "cudaStreamIsCapturing");
     if (cs != cudaStreamCaptureStatusNone) return LBM_OK;
-    const void *key[10] = {(const void *)(size_t)ctx->gen, ctx->dX, ctx->dU, ctx->dOm, ctx->dR, ctx->dF,
+    // (the adjoint's tiles have minimum-image flags of their own)
+    const int *wr = ctx->g.wrap_img;
+    const void *key[10] = {(const void *)(size_t)(8 * ctx->gen + wr[0] + 2 * wr[1] + 4 * wr[2]), ctx->dX, ctx->dU, ctx->dOm, ctx->dR, ctx->dF,
                            ctx->dT, ctx->dFr, ctx->dPf, (const void *)(size_t)ctx->np};
-    const int a = ctx->cur, b = bin ? 1 : 0;
+    const int a = ctx->cur + 2 * ctx->keep, b = bin ? 1 : 0;
     bool same = ctx->sgraph[a][b] != NULL;
     for (int k = 0; same && k < 10; ++k) same = (ctx->sgkey[a][b][k] == key[k]);
     if (!same) {
@@ -612,7 +617,7 @@ static lbm_status ctx_step_graph(lbm_ctx *ctx, bool bin, bool *done) {
 static int ctx_step_kernels(const lbm_ctx *ctx, const bool deferred) {
     if (ctx->np == 0) return 1;
     if (open_faces(ctx->g)) return 3;
-    if (ctx->elem == 2) return ctx->dim == 2 ? 4 : 3;
+    if (ctx->elem == 2 || ctx->keep) return ctx->dim == 2 ? 4 : 3;
     return 2 + (deferred ? 1 : 0) + (may_overflow(ctx->p.tile_cap, ctx->np) ? 1 : 0);
 }
 

@@ -62,8 +62,9 @@ struct lbm_ctx {
     // one step replayed from a CUDA graph (by population parity and whether it bins),
     // keyed on what its kernels capture; `gen` changes with every call that changes the
     // parameters or buffers a step reads
-    cudaGraphExec_t sgraph[2][2];
-    const void *sgkey[2][2][10];
+    cudaGraphExec_t sgraph[4][2];      // [population buffer + 2 keep][binning]
+    const void *sgkey[4][2][10];
+    int keep;                  // the adjoint's steps (Tiles::keep, narrow tiles)
     long long gen;
     // one coupled step (fluid step + DEM call) replayed from a CUDA graph, by parity and
     // whether it bins, keyed on the fluid step's key, the DEM call's and the sub-step count

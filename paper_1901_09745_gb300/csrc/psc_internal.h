@@ -123,6 +123,7 @@ struct Tiles {
     int *stats;          // [0] tiles that overflowed cap, [1] largest count, [2] length of
                          // the overflow list, [3] [6] work counters of the 16-bit kernels over
                          // the fluid and the particle tiles (zero between launches), [4] tiles with candidates, [5] tiles without
+    int keep = 0;        // FP32: step by the kernels of 16-bit storage (see launch_collide_stream_l)
     int *work;           // work counters of the step's kernel (zero between launches): [0]
                          // blocks that left, then kCounters of them, a cache line each
     void *blocks;        // per-tile packed candidate records (compute type), see psc_kernels.cuh

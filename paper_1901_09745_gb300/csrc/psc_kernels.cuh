@@ -889,8 +889,8 @@ k_collide_overflow(const S *__restrict__ fin, S *__restrict__ fout, Geom g, Phys
         __syncthreads();
     }
     pdl_wait();
-    // the 16-bit kernel before this one has finished: clear its work counters
-    if (sizeof(S) == 2 && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) {
+    // the pair kernel before this one has finished: clear its work counters
+    if ((sizeof(S) == 2 || tl.keep) && blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) {
         tl.stats[3] = 0;
         tl.stats[6] = 0;
     }
@@ -1141,7 +1141,7 @@ cudaError_t launch_overflow(const void *fin, void *fout, const Geom &g, const Ph
         if (e != cudaSuccess) return e;
     }
     const dim3 block(L::TX, L::TY, L::TZ);
-    if (sizeof(S) != 2) return launch_pdl(okern, dim3(32), block, osmem, s, (const S *)fin, (S *)fout, g, pt, tl, pd, flags);
+    if (sizeof(S) != 2 && !tl.keep) return launch_pdl(okern, dim3(32), block, osmem, s, (const S *)fin, (S *)fout, g, pt, tl, pd, flags);
     okern<<<32, block, osmem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
     return cudaGetLastError();
 }
@@ -1214,8 +1214,9 @@ inline cudaError_t block_registers(K kern, int threads, int &regs) {
     return e;
 }
 
-// 16-bit storage. Without particles: the fluid kernel over every tile. With particles in 2D: the particle-tile kernel (4 blocks per SM) and
-// the fluid-tile kernel (3 blocks per SM) side by side on two streams, which together fill
+// 16-bit storage (and the adjoint's steps in FP32). Without particles: the fluid kernel over every
+// tile. With particles in 2D: the particle-tile kernel (4 blocks per SM) and the fluid-tile
+// kernel (3 blocks per SM) side by side on two streams, which together fill
 // each SM's register file, so the issue-bound particle tiles and the DRAM-bound fluid tiles
 // share every SM for the whole step; without a second stream, one after the other. In 3D
 // the particle-tile kernel holds all the registers an SM has, and takes the
@@ -1329,6 +1330,13 @@ cudaError_t launch_collide_stream_l(const void *fin, void *fout, const Geom &g, 
     if constexpr (sizeof(S) == 2) {
         return launch_collide_stream16<L, S, PSC>(fin, fout, g, ph, tl, pd, flags, s, ov);
     } else {
+        // The adjoint's objective is one number, a sum over cells that may cancel to next to nothing
+        // (128^3 with 200 spheres: 10 or 0.003 out of terms that add up to 200), so another order of
+        // FP32 roundings in the state shows in its fourth digit although it is no less exact. Its
+        // steps keep the order they had: 5.80 ms for 20 steps with gradient where k_step takes 5.41.
+        if constexpr (sizeof(S) == 4 && PSC == 0) {
+            if (tl.keep) return launch_collide_stream16<L, S, PSC>(fin, fout, g, ph, tl, pd, flags, s, ov);
+        }
         // pairs in one access: every row of every direction starts on a pair boundary
         const bool vec = g.n[0] % 2 == 0 && ((uintptr_t)fin | (uintptr_t)fout) % (2 * sizeof(S)) == 0;
         if constexpr (L::D == 3 && sizeof(S) == 4) {

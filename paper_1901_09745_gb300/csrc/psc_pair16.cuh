@@ -1,5 +1,5 @@
-// psc_pair16.cuh -- the collide-stream step of lattices stored in 16 bits (included by
-// psc_kernels.cuh inside namespace psc, after psc_pair.cuh).
+// psc_pair16.cuh -- the collide-stream step of lattices stored in 16 bits, and the FP32 steps of the
+// adjoint (included by psc_kernels.cuh inside namespace psc, after psc_pair.cuh).
 //
 // A 128-thread block owns one tile (32 x 8 cells in 2D, 32 x 4 x 2 in 3D). Each warp takes
 // two rows of it (2D: rows 2w and 2w + 1; 3D: row w at both z), each lane the two cells of
@@ -18,7 +18,8 @@
 // rounded to 16 bits, a few in ten thousand come out one unit apart, and after some ten steps the
 // rounding of the whole state has nothing in common with the earlier one. It is as accurate
 // (forces on 5563 spheres after 10 steps of 256^3: 3.2e-5 off FP64 both ways) and faster (756 ->
-// 500 us), but a run's 16-bit results would not be those it gave before.
+// 500 us), but a run's 16-bit results would not be those it gave before. (The adjoint in FP32:
+// see launch_collide_stream_l.)
 
 namespace h16 {
 

@@ -323,8 +323,8 @@ const char *lbm_decomp_last_error(const lbm_decomp *d);                  /* neve
  * PSC collision, pull streaming, force and torque) on buffers the caller owns, and
  * allocates nothing: no cudaMalloc, no cudaFree, no host heap. Its working memory (tile
  * candidate lists and packed records, f(r) per particle, flag words) is one fixed array of
- * LBM_NOALLOC_SCRATCH_BYTES bytes that lives in the library image on every GPU that loads
- * the library, until the process exits. A lattice/particle set needing more working memory
+ * LBM_NOALLOC_SCRATCH_BYTES bytes (and 8 KB of work counters) that lives in the library
+ * image on every GPU that loads the library, until the process exits. A lattice/particle set needing more working memory
  * than that is rejected with LBM_ERR_ARG and a message from lbm_noalloc_last_error().
  *
  *   p       lattice, extent, bc, tau, body force, storage, psc, shell_h, dev_scale as for

@@ -5,8 +5,8 @@
  * JKR contact-radius solve, displacement since the neighbour list's build) and the host
  * checks of a particle upload. These calls run the same source on the host, so tests can check
  * the compiled arithmetic against brute force without a GPU. They allocate nothing, touch no
- * device and never fail; arguments are plain values and caller-owned arrays. Not part of the
- * simulation interface of psc_lbm.h. */
+ * device and never fail; arguments are plain values and caller-owned arrays. One more entry,
+ * psc_test_fill_work, writes to a device. Not part of the simulation interface of psc_lbm.h. */
 #ifndef PSC_TESTING_H
 #define PSC_TESTING_H
 
@@ -39,16 +39,22 @@ int psc_test_contact_sign(double d2, double S, int *ge0, int *gt0);
 /* The JKR contact-radius solve (reading R14): s = sqrt(a / a0) for t = delta_N R / a0^2,
  * started from s_prev; *fail = 1 when it did not converge, *iters the converging iteration. */
 float psc_test_jkr_s(float t, float s_prev, int *fail, int *iters);
-/* The DEM's squared displacement test (FP32, one image shift on periodic axes) of a
- * particle at x[3] from its position xr[3] at the last neighbour-list build. */
 /* The kernels' integer forms of (float)v and (double)v. */
 float psc_test_to_f32(double v);
 double psc_test_to_f64(float v);
+/* The DEM's squared displacement test (FP32, one image shift on periodic axes) of a
+ * particle at x[3] from its position xr[3] at the last neighbour-list build. */
 float psc_test_moved2(const double *x, const double *xr, const int *n, const int *periodic, int dim);
 /* The host-side checks of a particle upload: 1 when the m values are all finite; the
  * smallest r^2 and the largest r over n radii. */
 int psc_test_all_finite(const double *a, long long m);
 void psc_test_radii_range(const double *R, int n, double *s2min, double *rmax);
+/* Fill the work counters of the step's kernel (those of ctx in order of its stream; of
+ * lbm_psc_step_noalloc on the current device when ctx is NULL, once it has been called there)
+ * with the byte value, as a launch that ended in mid-step might leave them: each step
+ * clears them itself. Returns 0, or -1 when there are none or CUDA fails. */
+struct lbm_ctx;
+int psc_test_fill_work(struct lbm_ctx *ctx, int value);
 
 #ifdef __cplusplus
 }

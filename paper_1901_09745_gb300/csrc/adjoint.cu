@@ -503,7 +503,7 @@ extern "C" lbm_status lbm_adjoint_backward(lbm_ctx *ctx, long long token, double
         scratch_parts.F = w.sF;
         scratch_parts.T = w.sT;
         if (n > 0 && !ctx->bins_valid) {
-            ACK(launch_clear(ctx->tile_count, ctx->ntiles, ctx->tile_stats, NULL, NULL, 0, ctx->stream), "clear tile counts");
+            ACK(launch_clear(tl.work, ctx->tile_count, ctx->ntiles, ctx->tile_stats, NULL, NULL, 0, ctx->stream), "clear tile counts");
             ACK(launch_bin(ctx->dim, ctx->g, ctx->ph, tl, scratch_parts, ctx->stream), "bin kernel");
             ACK(launch_pack(ctx->q, ctx->p.storage, ctx->g, tl, scratch_parts, ctx->ntiles, ctx->stream), "pack kernel");
         }
@@ -515,6 +515,7 @@ extern "C" lbm_status lbm_adjoint_backward(lbm_ctx *ctx, long long token, double
             ACK(cudaMemcpyAsync(w.seg, w.ckpt + w.popa * (size_t)sidx, w.pop, cudaMemcpyDeviceToDevice, ctx->stream),
                 "restore checkpoint");
             for (int t = t0 + 1; t < t1; ++t) {
+                if (n > 0 && !tl.keep) ACK(launch_clear(tl.work, NULL, 0, NULL, NULL, NULL, 0, ctx->stream), "clear counters");
                 ACK(launch_collide_stream(ctx->p.storage, ctx->q, w.seg + w.popa * (size_t)(t - 1 - t0),
                                           w.seg + w.popa * (size_t)(t - t0), ctx->g, ctx->ph, tl, scratch_parts,
                                           ctx->flags, ctx->stream, &ctx->ov),

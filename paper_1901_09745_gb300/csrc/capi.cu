@@ -243,7 +243,6 @@ extern "C" lbm_status lbm_create(const lbm_params *p, lbm_ctx **out) {
     if (e == cudaSuccess) e = cudaMalloc(&ctx->f[1], bytes);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->flags, 4 * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&ctx->step_work, kWorkWords * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemsetAsync(ctx->step_work, 0, kWorkWords * sizeof(int), ctx->stream);
     if (e == cudaSuccess) e = cudaHostAlloc((void **)&ctx->hflags, 4 * sizeof(int), cudaHostAllocMapped);
     if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&ctx->hflags_dev, ctx->hflags, 0);
     // rest state f_i = w_i: every stored deviation is zero (all-zero bits in every format)
@@ -555,7 +554,7 @@ extern "C" lbm_status lbm_set_particles(lbm_ctx *ctx, int n, const double *X, co
 // Queue the binning of the particles into the tiles' candidate lists (no host state).
 static lbm_status ctx_enqueue_bin(lbm_ctx *ctx) {
     Tiles tl = ctx_tiles(ctx);
-    CK(launch_clear(ctx->tile_count, ctx->ntiles, ctx->tile_stats, NULL, NULL, 0, ctx->stream), "clear tile counts");
+    CK(launch_clear(ctx->step_work, ctx->tile_count, ctx->ntiles, ctx->tile_stats, NULL, NULL, 0, ctx->stream), "clear tile counts");
     CK(launch_bin(ctx->dim, ctx->g, ctx->ph, tl, ctx_parts(ctx), ctx->stream), "bin kernel");
     CK(launch_pack(ctx->q, ctx->p.storage, ctx->g, tl, ctx_parts(ctx), ctx->ntiles, ctx->stream), "pack kernel");
     return LBM_OK;
@@ -569,7 +568,7 @@ static lbm_status ctx_enqueue_step(lbm_ctx *ctx, bool bin, cudaEvent_t *ev) {
             lbm_status st = ctx_enqueue_bin(ctx);
             if (st != LBM_OK) return st;
         } else {
-            CK(launch_clear(NULL, 0, NULL, ctx->dF, ctx->dT, 3LL * ctx->np, ctx->stream), "clear F and T");
+            CK(launch_clear(ctx->step_work, NULL, 0, NULL, ctx->dF, ctx->dT, 3LL * ctx->np, ctx->stream), "clear F and T");
         }
     }
     if (ev) CK(cudaEventRecord(ev[0], ctx->stream), "cudaEventRecord");

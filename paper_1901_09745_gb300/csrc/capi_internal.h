@@ -87,6 +87,7 @@ lbm_status ctx_bin(lbm_ctx *ctx);
 lbm_status ctx_step_once(lbm_ctx *ctx);
 psc::Parts ctx_parts(lbm_ctx *ctx);
 void ctx_update_wrap(lbm_ctx *ctx);
+int noalloc_fill_work(int value);      // psc_testing.h's psc_test_fill_work without a context
 lbm_status ctx_check_radii(lbm_ctx *ctx, const double *R, int n);
 lbm_status ctx_reserve_particles(lbm_ctx *ctx, int n);
 void dem_release(dem_ctx *dem);

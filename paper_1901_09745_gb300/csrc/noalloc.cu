@@ -29,8 +29,8 @@ constexpr int kNoAllocCap = 16;        // candidate records per tile (more take 
 constexpr int kMaxDevices = 64;
 constexpr size_t kWorkBytes = (size_t)psc::kWorkWords * sizeof(int);
 
-// the step's work counters lie behind the declared size
-static __device__ __align__(256) unsigned char g_scratch[kScratchBytes + kWorkBytes];
+// the step's work counters, then the declared size
+static __device__ __align__(256) unsigned char g_scratch[kWorkBytes + kScratchBytes];
 
 // Device address of g_scratch for each device, looked up once (with that device current),
 // and the second stream and events of the 2D step on that device, created at the same time.
@@ -144,7 +144,7 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
     if (dev < 0 || dev >= kMaxDevices) return fail(LBM_ERR_UNSUPPORTED, "device index out of range");
-    unsigned char *base;
+    unsigned char *work, *base;
     {
         std::lock_guard<std::mutex> lock(g_setup_mutex);
         if (!g_scratch_addr[dev]) {
@@ -158,7 +158,8 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
                 cudaEventCreateWithFlags(&ov.join, cudaEventDisableTiming) == cudaSuccess)
                 g_overlap[dev] = ov;     // else the kernels of a step share one stream
         }
-        base = (unsigned char *)g_scratch_addr[dev];
+        work = (unsigned char *)g_scratch_addr[dev];
+        base = work + kWorkBytes;
     }
 
     cudaStream_t s = (cudaStream_t)p->stream;
@@ -169,16 +170,15 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
     tl.cap = kNoAllocCap;
     tl.blocks = base + o_blocks;
     tl.order = (unsigned *)(base + o_order);
-    tl.work = (int *)(base + kScratchBytes);
+    tl.work = (int *)work;
     int *flags = (int *)(base + o_flags);
     Parts pd;
     pd.n = n; pd.X = X; pd.U = U; pd.Om = Omega; pd.R = radius; pd.Fr = (double *)(base + o_fr);
     pd.F = F; pd.T = T;
     pd.Pf = nullptr;
 
-    // what must start at zero: tile counts, stats, flags (the rest is fully rewritten; the work
-    // counters are zero from the start, and each launch leaves them so)
-    e = cudaMemsetAsync(base, 0, o_list, s);
+    // what must start at zero: work counters, tile counts, stats, flags (the rest is fully rewritten)
+    e = cudaMemsetAsync(work, 0, kWorkBytes + o_list, s);
     if (e == cudaSuccess && n > 0) e = launch_f_of_r(is2d ? 2 : 3, radius, (double *)(base + o_fr), n, s);
     if (e == cudaSuccess && n > 0) e = launch_bin(is2d ? 2 : 3, g, ph, tl, pd, s);
     if (e == cudaSuccess && n > 0) e = launch_pack(p->lattice, p->storage, g, tl, pd, ntiles, s);
@@ -187,6 +187,16 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
                                   g_overlap[dev].join ? &g_overlap[dev] : nullptr);
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
     return LBM_OK;
+}
+
+// (psc_testing.h, for ctx = NULL)
+int noalloc_fill_work(int value) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices || !g_scratch_addr[dev]) return -1;
+    cudaError_t e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemset(g_scratch_addr[dev], value, kWorkBytes);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    return e == cudaSuccess ? 0 : -1;
 }
 
 // the bounds-check word of this translation unit (see psc_internal.h)

@@ -10,12 +10,13 @@
 
 namespace psc {
 
-// What a step accumulates into, cleared: the tiles' counts and statistics before a binning, F and T
-// before a step that keeps its lists. One launch (whose successor starts beside it) where two
-// memsets stood: 1.5 us or so of a step.
-__global__ void k_clear(int *count, long long ntiles, int *stats, double *F, double *T, long long m) {
+// What a step accumulates into, cleared: the work counters of its kernel, the tiles' counts and
+// statistics before a binning, F and T before a step that keeps its lists. One launch (whose
+// successor starts beside it) where two memsets stood: 1.5 us or so of a step.
+__global__ void k_clear(int *work, int *count, long long ntiles, int *stats, double *F, double *T, long long m) {
     pdl_launch();
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    if (t < kWorkWords / kCounterStride) work[t * kCounterStride] = 0;
     for (long long k = t; k < ntiles; k += step) count[k] = 0;
     for (long long k = t; k < m; k += step) { F[k] = 0.0; T[k] = 0.0; }
     if (stats && t < kTileStats) stats[t] = 0;
@@ -160,10 +161,12 @@ __global__ void k_download(const double *F, const double *T, double *Fo, double 
     if (k < 4) flags_out[k] = flags[k];
 }
 
-cudaError_t launch_clear(int *count, long long ntiles, int *stats, double *F, double *T, long long m, cudaStream_t s) {
+cudaError_t launch_clear(int *work, int *count, long long ntiles, int *stats, double *F, double *T, long long m,
+                         cudaStream_t s) {
     const int threads = 256;
-    const long long work = ntiles > m ? ntiles : m, blocks = (work + threads - 1) / threads;
-    k_clear<<<(unsigned)(blocks < 1 ? 1 : (blocks > 1024 ? 1024 : blocks)), threads, 0, s>>>(count, ntiles, stats, F, T, m);
+    const long long words = ntiles > m ? ntiles : m, blocks = (words + threads - 1) / threads;
+    k_clear<<<(unsigned)(blocks < 1 ? 1 : (blocks > 1024 ? 1024 : blocks)), threads, 0, s>>>(work, count, ntiles, stats, F, T,
+                                                                                              m);
     return cudaGetLastError();
 }
 

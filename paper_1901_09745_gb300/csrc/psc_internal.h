@@ -124,8 +124,10 @@ struct Tiles {
                          // the overflow list, [3] [6] work counters of the 16-bit kernels over
                          // the fluid and the particle tiles (zero between launches), [4] tiles with candidates, [5] tiles without
     int keep = 0;        // FP32: step by the kernels of 16-bit storage (see launch_collide_stream_l)
-    int *work;           // work counters of the step's kernel (zero between launches): [0]
-                         // blocks that left, then kCounters of them, a cache line each
+    int *work;           // work counters of the step's kernel over the lists of tiles, a cache
+                         // line each: kCounters for a launch over both lists or that of the tiles
+                         // with candidates, then as many for one over the tiles without. Cleared
+                         // before each step (launch_clear), in an earlier kernel
     void *blocks;        // per-tile packed candidate records (compute type), see psc_kernels.cuh
     unsigned *order;     // [3 * ntiles] tile numbers: tiles with candidates, then (from ntiles
                          // on) tiles without, then (from 2 ntiles on) tiles with more than
@@ -133,7 +135,7 @@ struct Tiles {
 };
 constexpr int kTileStats = 8;
 constexpr int kCounters = 32, kCounterStride = 32;
-constexpr int kWorkWords = (1 + kCounters) * kCounterStride;
+constexpr int kWorkWords = 2 * kCounters * kCounterStride;
 
 // Particle state on the device (FP64), and the force/torque accumulators (Eq. 14).
 struct Parts {
@@ -173,13 +175,14 @@ cudaError_t launch_gather(int storage, int lattice, const void *fin, double *f_o
 // Overwrite the state from pre-collision populations (inverse of the pull).
 cudaError_t launch_set(int storage, int lattice, const double *f, void *fout,
                        const Geom &g, const Phys &ph, cudaStream_t s);
-// Bin particles into tile candidate lists and zero F, T.
 // Candidates a tile may have in the step's usual kernels; tiles with more overflow, which takes more
 // particles (no particle is on a tile's list twice).
 constexpr int kPairCap = 32;
 __host__ inline bool may_overflow(const int cap, const int n) { return n > (cap < kPairCap ? cap : kPairCap); }
-// Clear ntiles counts (and stats unless null) and m values of F and T each.
-cudaError_t launch_clear(int *count, long long ntiles, int *stats, double *F, double *T, long long m, cudaStream_t s);
+// Clear the step's work counters, ntiles counts (and stats unless null) and m values of F and T each.
+cudaError_t launch_clear(int *work, int *count, long long ntiles, int *stats, double *F, double *T, long long m,
+                         cudaStream_t s);
+// Bin particles into tile candidate lists and zero F, T.
 cudaError_t launch_bin(int dim, const Geom &g, const Phys &ph, const Tiles &tl,
                        const Parts &pd, cudaStream_t s);
 // Sort each tile's list and write its packed candidate records (in the storage's compute type).

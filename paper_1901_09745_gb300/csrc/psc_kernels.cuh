@@ -1152,7 +1152,7 @@ cudaError_t launch_overflow(const void *fin, void *fout, const Geom &g, const Ph
 // caller's kernels find no room beside them).
 constexpr int kDeferF = 3;
 
-// One launch of the step's kernel over the tiles of kind `which` (blocks_per_sm > 0 limits it).
+// One launch of the step's kernel over the lists `which` (blocks_per_sm > 0 limits it).
 template <class L, typename S, int PSC, bool SOLID, bool VEC>
 cudaError_t launch_step_t(const void *fin, void *fout, const Geom &g, const PhysT<typename Store<S>::T> &pt,
                           const Tiles &tl, const Parts &pd, int *flags, int which, int blocks_per_sm, cudaStream_t s) {
@@ -1173,10 +1173,26 @@ cudaError_t launch_step_t(const void *fin, void *fout, const Geom &g, const Phys
     if (e != cudaSuccess) return e;
     if (blocks_per_sm > 0 && nb > (unsigned)(blocks_per_sm * sms)) nb = (unsigned)(blocks_per_sm * sms);
     const Dirs<L, S> f(fin, fout, g);
-    if (which != kFluidTiles)      // (on the second stream after an event: the usual order)
+    if (which != kFluidTiles)
         return launch_pdl(kern, dim3(nb), dim3((unsigned)threads), 0, s, f, g, pt, tl, pd, flags, tl.work, which, shift);
-    kern<<<nb, threads, 0, s>>>(f, g, pt, tl, pd, flags, tl.work, which, shift);
+    // on the second stream after an event: the usual order, and counters of its own
+    kern<<<nb, threads, 0, s>>>(f, g, pt, tl, pd, flags, tl.work + kCounters * kCounterStride, which, shift);
     return cudaGetLastError();
+}
+
+// The step of a lattice without particles; few units go to blocks of one warp, spread over the SMs.
+template <class L, typename S, bool VEC>
+cudaError_t launch_fluid_t(const void *fin, void *fout, const Geom &g, const PhysT<typename Store<S>::T> &pt, int *flags,
+                           cudaStream_t s) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    static_assert(kUnits % kPWarps == 0, "a block's units end with the lattice's");
+    const long long units = (long long)g.nt[0] * g.nt[1] * g.nt[2] * kUnits;
+    const int threads = units <= 8LL * sms ? 32 : kPThreads;
+    return launch_pdl(k_fluid<L, S, VEC>, dim3((unsigned)(units / (threads / 32))), dim3((unsigned)threads), 0, s,
+                      Dirs<L, S>(fin, fout, g), g, pt, flags);
 }
 
 // One collide-stream step. Without particles: the fluid kernel over every tile. With
@@ -1190,7 +1206,7 @@ cudaError_t launch_collide_stream_t(const void *fin, void *fout, const Geom &g, 
                                     Overlap *ov) {
     using T = typename Store<S>::T;
     const PhysT<T> pt = make_phys<T>(ph, L::Q);
-    if (pd.n == 0) return launch_step_t<L, S, 0, false, VEC>(fin, fout, g, pt, tl, pd, flags, kAllTiles, 0, s);
+    if (pd.n == 0) return launch_fluid_t<L, S, VEC>(fin, fout, g, pt, flags, s);
     const bool defer = ov && ov->aux && ov->defer && L::D == 2 && sizeof(T) == 4;
     cudaError_t e = launch_step_t<L, S, PSC, true, VEC>(fin, fout, g, pt, tl, pd, flags,
                                                               defer ? kParticleTiles : kBothLists, 0, s);

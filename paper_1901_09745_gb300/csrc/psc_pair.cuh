@@ -569,21 +569,29 @@ __device__ __forceinline__ void unit_step(const UnitPos<L> &up, const int cnt,
     }
 }
 
-// Which tiles a launch takes.
+// Which lists of tiles a launch takes.
 enum StepTiles {
-    kAllTiles = 0,         // every tile by its number (no particles, no lists)
     kParticleTiles = 1,    // the list of tiles with candidates
     kFluidTiles = 2,       // the list of tiles without
     kBothLists = 3         // those with candidates first
 };
 
-// One collide-stream step over tiles of kind `which`: persistent warps, an item being a tile or
-// (shift > 0) one of 1 << shift equal parts of its units. Items go through work counters (they
-// differ in cost, and so do SMs in their distance from memory), kCounters of them, a block's warps
-// sharing one, since a single counter's atomics would take as long as the step of a 2D lattice.
-// An item's number is fetched two items ahead of its turn, its tile one. The last block to leave
-// clears the counters for the next launch. Tiles with more than kPairCap candidates are left to
-// k_collide_overflow.
+// First cell of a tile.
+template <class L> __device__ __forceinline__ void unit_origin(const Geom &g, const unsigned tile, UnitPos<L> &u) {
+    const unsigned t1 = tile / (unsigned)g.nt[0], tz = t1 / (unsigned)g.nt[1];
+    u.x0 = (int)(tile - t1 * (unsigned)g.nt[0]) * L::TX;
+    u.y0 = (int)(t1 - tz * (unsigned)g.nt[1]) * L::TY;
+    u.z0 = (int)tz * L::TZ;
+}
+
+// One collide-stream step over the tiles of the lists `which`: persistent warps, an item being a
+// tile or (shift > 0) one of 1 << shift equal parts of its units. Items go through work counters
+// (they differ in cost, and so do SMs in their distance from memory), kCounters of them, a block's
+// warps sharing one, since a single counter's atomics would take as long as the step of a 2D
+// lattice. An item's number is fetched two items ahead of its turn, its tile one. The counters
+// are cleared by an earlier kernel (k_clear): at the end of this one, the last fetch of a warp, which
+// nothing waits for, might land after a clearing store of another. Tiles with more than kPairCap
+// candidates are left to k_collide_overflow.
 //
 // Blocks per SM (registers): more or fewer measured slower (3D FP32 with 5 instead of 4: 256^3 with
 // 2000 spheres 567 us against 431, with 3: 541 against 512 on narrow tiles).
@@ -602,18 +610,17 @@ k_step(const __grid_constant__ Dirs<L, S> f, const __grid_constant__ Geom g,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned ntiles = (unsigned)g.nt[0] * (unsigned)g.nt[1] * (unsigned)g.nt[2];
     const unsigned np = (SOLID && (which & kParticleTiles)) ? (unsigned)tl.stats[4] : 0u;
-    const unsigned nlist = which == kAllTiles ? ntiles : np + ((which & kFluidTiles) ? (unsigned)tl.stats[5] : 0u);
+    const unsigned nlist = np + ((which & kFluidTiles) ? (unsigned)tl.stats[5] : 0u);
     const long long nitem = (long long)nlist << shift;       // 1 << shift items a tile
     const int units = kUnits >> shift;
     const int groups = min(kCounters, (int)gridDim.x), group = blockIdx.x % groups;
-    int *const counter = work + (1 + group) * kCounterStride;
+    int *const counter = work + group * kCounterStride;
     auto fetch = [&]() { return lane == 0 ? atomicAdd(counter, 1) : 0; };       // lane 0's, not waited for
     auto number = [&](const int raw) { return (long long)__shfl_sync(kFull, raw, 0) * groups + group; };
     // the tile of an item (a load for lists)
     auto tile_of = [&](const long long it) {
         if (it >= nitem) return 0u;
         const unsigned ti = (unsigned)(it >> shift);
-        if (which == kAllTiles) return ti;
         return (unsigned)PSC_IDX(tl.order[ti < np ? ti : ntiles + (ti - np)], ntiles, CHK_TILE);
     };
     const T *const blocks = reinterpret_cast<const T *>(tl.blocks);
@@ -626,10 +633,7 @@ k_step(const __grid_constant__ Dirs<L, S> f, const __grid_constant__ Geom g,
         raw = fetch();
         const unsigned ntile = tile_of(nx);
         UnitPos<L> u;
-        const unsigned t1 = tile / (unsigned)g.nt[0], tz = t1 / (unsigned)g.nt[1];
-        u.x0 = (int)(tile - t1 * (unsigned)g.nt[0]) * L::TX;
-        u.y0 = (int)(t1 - tz * (unsigned)g.nt[1]) * L::TY;
-        u.z0 = (int)tz * L::TZ;
+        unit_origin<L>(g, tile, u);
         const int k0 = (int)(it & ((1 << shift) - 1)) * units;
         const int cnt = (SOLID && it < ((long long)np << shift)) ? tl.count[tile] : 0;
         const T *const recs = blocks + (size_t)tile * block_elems<T>(tl.cap) + head_elems<T>();
@@ -641,9 +645,20 @@ k_step(const __grid_constant__ Dirs<L, S> f, const __grid_constant__ Geom g,
         }
         it = nx; tile = ntile;
     }
-    __syncthreads();
-    if (threadIdx.x == 0 && atomicAdd(work, 1) == (int)gridDim.x - 1) {
-        for (int k = 0; k < kCounters; ++k) work[(1 + k) * kCounterStride] = 0;
-        work[0] = 0;
-    }
+}
+
+// One step of a lattice without particles: no lists, so a unit per warp in the order of the blocks
+// and no counters to share out. Bound by DRAM: 2048^2 FP32 47.6 us, 256^3 367 (the state once 44 and
+// 376 at the copy's rate); warps that drew their units from counters took 54 and 381.
+template <class L, typename S, bool VEC>
+__global__ void __launch_bounds__(kPThreads, (step_blocks<L, S>()))
+k_fluid(const __grid_constant__ Dirs<L, S> f, const __grid_constant__ Geom g,
+        const __grid_constant__ PhysT<typename Store<S>::T> ph, int *flags) {
+    pdl_wait();
+    pdl_launch();
+    const unsigned it = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    UnitPos<L> u;
+    unit_origin<L>(g, it / kUnits, u);
+    u.k = (int)(it % kUnits);
+    unit_step<L, S, 0, false, VEC>(u, 0, nullptr, f, g, ph, Parts{}, flags, nullptr);
 }

@@ -1,7 +1,8 @@
 // testing.cu -- host entry points onto the __host__ __device__ helpers of hostdev.cuh, so
 // that the CPU tests check the arithmetic the kernels compile rather than a copy of it (see
-// include/psc_testing.h). Nothing here touches a GPU.
+// include/psc_testing.h). Nothing here but psc_test_fill_work touches a GPU.
 #include "../../include/psc_testing.h"
+#include "capi_internal.h"
 #include "hostcheck.h"
 #include "hostdev.cuh"
 
@@ -60,3 +61,7 @@ extern "C" float psc_test_moved2(const double *x, const double *xr, const int *n
     return moved2(x, xr, n, periodic, dim);
 }
 
+extern "C" int psc_test_fill_work(lbm_ctx *ctx, int value) {
+    if (!ctx) return noalloc_fill_work(value);
+    return cudaMemsetAsync(ctx->step_work, value, kWorkWords * sizeof(int), ctx->stream) == cudaSuccess ? 0 : -1;
+}

@@ -958,10 +958,12 @@ __device__ __noinline__ void moments_f64_cold(const T *df, double &drho, double 
 // The same sums from FP32 values, no less accurate than in FP64 but almost all on the FP32
 // pipe (error-free vector transformation of Rump, Ogita and Oishi, "Accurate floating-point
 // summation", 2008): with max |d| < 2^k every d is cut into q1 + q2 + r, q1 a multiple of
-// 2^(k-17), q2 of 2^(k-34), |r| <= 2^(k-35), by adding and subtracting 2^(k+7) and 2^(k-10).
+// 2^(k-17), q2 of 2^(k-34), |r| <= 2^(k-34), by adding and subtracting 2^(k+7) and 2^(k-10).
 // The at most 19 q1 of a sum (and likewise the q2) have an exact FP32 sum, whatever the signs;
-// the r's sum is rounded in FP32 at 2^(k-55). Two FP64 additions put a moment together.
-// Returns false, with nothing written, for values outside [2^-60, 2^10] (or not finite).
+// the r's sum, below 2^(k-29), is rounded in FP32 by at most 2^(k-54) an addition. Two FP64
+// additions put a moment together. rhof is the density with three roundings in FP32 (all three
+// parts count where it is far below 1: without the q2, a density of 0.02 was off by 1e-4 of itself
+// and the velocity by 2e-13). Returns false, with nothing written, for values outside [2^-60, 2^10] (or not finite).
 template <class L>
 __device__ __forceinline__ bool moments_split(const float *df, double &drho, double *j, float &rhof) {
     float m = 0.0f;
@@ -990,15 +992,15 @@ __device__ __forceinline__ bool moments_split(const float *df, double &drho, dou
 #pragma unroll
     for (int c = 0; c < 4; ++c) o[c] = (c <= L::D) ? (widen(t[0][c]) + widen(t[1][c])) + widen(t[2][c]) : 0.0;
     drho = o[0]; j[0] = o[1]; j[1] = o[2]; j[2] = o[3];
-    rhof = 1.0f + t[0][0];
+    rhof = 1.0f + __fadd_rn(__fadd_rn(t[0][0], t[1][0]), t[2][0]);
     return true;
 }
 
 // Density and force-shifted velocity (Eq. 5) of every cell in FP64, one block per lattice
 // tile, one warp per row. Bound by the FP64 pipe (1/64 of the FP32 rate): the moments of FP32
 // values are summed by moments_split, and u = (j + F/2) / rho shares one reciprocal (one
-// Newton step on the FP32 one, then per component the quotient and one residual correction,
-// which leaves it correctly rounded but for rare ties): 23 FP64 operations a cell where 19
+// Newton step on the FP32 one, off by at most 2^-18 for densities above 2^-6, then per component the
+// quotient and one residual correction, which leaves it correctly rounded but for rare ties): 23 FP64 operations a cell where 19
 // conversions, 95 additions and three divisions stood before. The three components leave
 // through shared memory, a row's 96 doubles in order. 256^3 D3Q19: 4.03 -> 0.82 ms in FP32,
 // 5.65 -> 0.82 ms in FP16 (its bytes take 0.27 and 0.17 ms); 2048^2 D2Q9 FP32: 0.66 -> 0.20 ms.

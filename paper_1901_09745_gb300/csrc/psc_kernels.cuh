@@ -897,10 +897,13 @@ k_collide_overflow(const S *__restrict__ fin, S *__restrict__ fout, Geom g, Phys
 }
 
 // Contexts with an open, inlet or outlet face, by the single-cell path whose pull classifies each
-// face (blocks striding over the tiles): SOLID the list of tiles with candidates, else those
-// without (every tile when there are no particles). Apart, the tiles without need a third of
-// the registers, so three blocks instead of one share an SM: a box of 120 x 60 x 60 with one
-// sphere takes 65 us a step where one kernel for both took 104.
+// face: SOLID the list of tiles with candidates (blocks striding over it), else those without
+// (every tile when there are no particles; a block each). Apart, the tiles without need a third of
+// the registers, so three blocks instead of one share an SM. Few tiles with candidates leave most
+// of the chip idle, so the other launch starts as soon as this one's blocks have (its tiles are
+// others) and ends after it; a block per tile evens out the SMs where those still run. A step of
+// 120 x 60 x 60 FP32 with one sphere: one kernel for both 104 us, one after the other 66, now 51
+// (58 with striding blocks); 500 x 300 FP64 with one disc 90, 105 and 88 (94).
 template <class L, typename S, int PSC, bool SOLID>
 __global__ void __launch_bounds__(kThreads, SOLID ? 1 : (sizeof(S) == 8 ? 2 : 3))
 k_collide_faces(const S *__restrict__ fin, S *__restrict__ fout, Geom g, PhysT<typename Store<S>::T> ph,
@@ -909,12 +912,14 @@ k_collide_faces(const S *__restrict__ fin, S *__restrict__ fout, Geom g, PhysT<t
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long s_mask[kWarps];
     const unsigned ntiles = (unsigned)g.nt[0] * (unsigned)g.nt[1] * (unsigned)g.nt[2];
+    if (SOLID) pdl_launch();      // what both read was there before this launch, and their tiles differ
     const unsigned n = SOLID ? (unsigned)tl.stats[4] : (pd.n > 0 ? (unsigned)tl.stats[5] : ntiles);
     for (unsigned it = blockIdx.x; it < n; it += gridDim.x) {
         const unsigned tile = SOLID ? tl.order[it] : (pd.n > 0 ? tl.order[ntiles + it] : it);
         psc_tile<L, S, PSC, true, !SOLID>(tile, fin, fout, g, ph, tl, pd, flags, reinterpret_cast<T *>(smem), s_mask);
         __syncthreads();
     }
+    if (!SOLID) pdl_wait();       // not done before the other is
 }
 
 // ---------------------------------------------------------------- gather / set kernels
@@ -1335,9 +1340,8 @@ cudaError_t launch_faces_t(const void *fin, void *fout, const Geom &g, const Phy
         kern<<<nb, block, smem, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
     }
     auto kern = k_collide_faces<L, S, PSC, false>;
-    cudaError_t e = persistent_blocks(kern, 0, ntiles, nb, kThreads);
-    if (e != cudaSuccess) return e;
-    kern<<<nb, block, 0, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
+    if (pd.n > 0) return launch_pdl(kern, dim3((unsigned)ntiles), block, 0, s, (const S *)fin, (S *)fout, g, pt, tl, pd, flags);
+    kern<<<(unsigned)ntiles, block, 0, s>>>((const S *)fin, (S *)fout, g, pt, tl, pd, flags);
     return cudaGetLastError();
 }
 

@@ -835,7 +835,7 @@ __global__ void __launch_bounds__(kSubThreads, 6) k_dem_substep3(DemGeom g, DemP
         }
         // the contacts of the pass, added in slot order by the lane of each component
         if (!__any_sync(kFullMask, contact)) continue;
-        const unsigned group = G == 32 ? kFullMask : ((1u << (G & 31)) - 1u) << first;
+        const unsigned group = ((1u << G) - 1u) << first;
         unsigned m0 = __ballot_sync(kFullMask, contact && !odd) & group;      // orders the stores above, too
         unsigned m1 = __ballot_sync(kFullMask, contact && odd) & group;
         __syncwarp();

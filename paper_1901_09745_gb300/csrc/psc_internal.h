@@ -80,11 +80,11 @@ __host__ __device__ inline bool open_faces(const Geom &g) {
     for (int a = 0; a < 3; ++a) any |= face_kind(g, a, 0) >= FACE_OPEN || face_kind(g, a, 1) >= FACE_OPEN;
     return any;
 }
-// Tile extent along axis ax: 32 x 8 x 1 cells for D2Q9, 32 x 4 x 2 for D3Q19; wide tiles 64 x 4 x 1
-// and 64 x 2 x 2. One tile is one thread block of the single-cell kernels.
+// Tile extent along axis ax: 32 x 8 x 1 cells for D2Q9, 32 x 4 x 2 for D3Q19, wide tiles (D3Q19 only)
+// 64 x 2 x 2. One tile is one thread block of the single-cell kernels.
 __host__ __device__ inline int tile_ext(const int dim, const int wide, const int ax) {
     if (ax == 0) return wide ? 64 : 32;
-    if (ax == 1) return (dim == 2 ? 8 : 4) >> wide;
+    if (ax == 1) return dim == 2 ? 8 : (wide ? 2 : 4);
     return dim == 2 ? 1 : 2;
 }
 __host__ inline long long tile_number(const int dim, const int wide, const Geom &g) {

@@ -192,14 +192,10 @@ pull_one(const S *__restrict__ fin, const Geom &g, int x, int y, int z, long lon
 // as 0, `from_inlet` or `from_outlet` set) and is filled in by inflow_nebb or outlet_nebb
 // once all are pulled. A wall takes precedence over the inlet and outlet faces, these over
 // open faces.
-template <class L, typename S, bool RAW = false>
+template <class L, typename S>
 __device__ __forceinline__ typename Store<S>::T
 pull_one_faces(const S *__restrict__ fin, const Geom &g, int x, int y, int z, long long cell, int i,
                float2 sc, bool &from_inlet, bool &from_outlet) {
-    auto ld = [&](long long k) {
-        const long long c = PSC_IDX(k, L::Q * g.ncell, CHK_POP);
-        return RAW ? Store<S>::ldr(fin, c) : Store<S>::ld(fin, c, sc);
-    };
     int s[3] = {x - L::ex(i), y - L::ey(i), z - L::ez(i)};
     bool bounce = false, inflow = false, outflow = false;
 #pragma unroll
@@ -213,17 +209,17 @@ pull_one_faces(const S *__restrict__ fin, const Geom &g, int x, int y, int z, lo
             else outflow = true;
         }
     }
-    if (bounce) return ld((long long)opp<L>(i) * g.ncell + cell);
+    if (bounce) return Store<S>::ld(fin, PSC_IDX((long long)opp<L>(i) * g.ncell + cell, L::Q * g.ncell, CHK_POP), sc);
     from_inlet = inflow;
     from_outlet = outflow && !inflow;
     if (inflow || outflow) return (typename Store<S>::T)0;
     long long src = (long long)s[0] + (long long)g.n[0] * ((long long)s[1] + (long long)g.n[1] * s[2]);
-    return ld((long long)i * g.ncell + src);
+    return Store<S>::ld(fin, PSC_IDX((long long)i * g.ncell + src, L::Q * g.ncell, CHK_POP), sc);
 }
 
 // All Q populations of cell (x, y, z) after streaming, one pull_one per direction, the
 // unknown ones at an inlet filled in.
-template <class L, typename S, bool RAW = false>
+template <class L, typename S>
 __device__ __forceinline__ void pull_all(const S *__restrict__ fin, const Geom &g, int x, int y, int z,
                                          long long cell, const PhysT<typename Store<S>::T> &ph,
                                          typename Store<S>::T *df) {
@@ -231,12 +227,12 @@ __device__ __forceinline__ void pull_all(const S *__restrict__ fin, const Geom &
 #pragma unroll
     for (int i = 0; i < L::Q; ++i) {
         bool in = false, out = false;
-        df[i] = pull_one_faces<L, S, RAW>(fin, g, x, y, z, cell, i, ph.sc, in, out);
+        df[i] = pull_one_faces<L, S>(fin, g, x, y, z, cell, i, ph.sc, in, out);
         if (in) fill |= 1u << i;
         if (out) fillo |= 1u << i;
     }
-    if (fill) inflow_nebb<L, RAW>(df, ph, ph.sc, fill);
-    if (fillo) outlet_nebb<L, RAW>(df, ph, ph.sc, fillo);
+    if (fill) inflow_nebb<L, false>(df, ph, ph.sc, fill);
+    if (fillo) outlet_nebb<L, false>(df, ph, ph.sc, fillo);
 }
 
 // Warp sum of NV values per lane (NV a power of two <= 32) in NV - 1 + 5 - log2(NV) shuffles
@@ -378,10 +374,9 @@ __device__ __forceinline__ void pull_q(const S *__restrict__ fin, const Geom &g,
 // packing kernel after binning: a 16-byte header whose first element is the tile's
 // candidate count, then up to `cap` records of RW values of the compute type, sorted by
 // particle index (so per-cell sums do not depend on the binning's atomic order). A record
-// holds the particle's position relative to the tile origin (minimum image), radius,
-// f(r) of Eq. 18, velocity, spin and index. The collide-stream kernel fetches a tile's
-// header and first kPre records in one coalesced round trip issued before its population
-// loads, so the candidate table costs no extra latency on the critical path.
+// holds the particle's position relative to the tile origin (minimum image; in wide tiles
+// to its middle along x), radius, f(r) of Eq. 18 (negative for a particle that moves or
+// spins), velocity, spin and index.
 constexpr int RW = 12;
 enum { R_PX = 0, R_PY, R_PZ, R_R, R_FR, R_UX, R_UY, R_UZ, R_OX, R_OY, R_OZ, R_ID };
 
@@ -1397,9 +1392,15 @@ cudaError_t launch_gather_storage(int lattice, const void *fin, double *f_out, d
                                   double *u, const Geom &g, const Phys &ph, cudaStream_t s) {
     using T = typename Store<S>::T;
     if (rho || u) {
-        cudaError_t e = lattice == 9 ? launch_macro_t<D2Q9, S>((const S *)fin, rho, u, g, ph, s)
-                      : g.wide ? launch_macro_t<D3Q19w, S>((const S *)fin, rho, u, g, ph, s)
-                                                    : launch_macro_t<D3Q19, S>((const S *)fin, rho, u, g, ph, s);
+        cudaError_t e = lattice == 9 ? launch_macro_t<D2Q9, S>((const S *)fin, rho, u, g, ph, s) : cudaSuccess;
+        if (lattice != 9) {
+            if constexpr (sizeof(S) == 4) {
+                e = g.wide ? launch_macro_t<D3Q19w, S>((const S *)fin, rho, u, g, ph, s)
+                           : launch_macro_t<D3Q19, S>((const S *)fin, rho, u, g, ph, s);
+            } else {
+                e = launch_macro_t<D3Q19, S>((const S *)fin, rho, u, g, ph, s);
+            }
+        }
         if (e != cudaSuccess || !f_out) return e;
     }
     const int threads = 256;

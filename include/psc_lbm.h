@@ -159,7 +159,8 @@ lbm_status lbm_set_body_force(lbm_ctx *ctx, const double *F);
  * paper has no adjoint; this is a derived quantity of Eq. 1-18). The particles must be
  * static (U = Omega = 0: LBM_ERR_UNSUPPORTED otherwise), storage FP32 or FP64, the
  * modified scheme, periodic or wall axes only, and every tile's candidates within tile_cap. Runs the T forward steps
- * (the context ends at step T as after lbm_step(ctx, T)), keeping a checkpoint every
+ * (the context ends at step T as after lbm_step(ctx, T), in FP32 up to rounding: the adjoint's
+ * FP32 steps add in an order of their own), keeping a checkpoint every
  * checkpoint_every steps, then the reverse sweep, re-running each segment forward. The
  * gradient is exact for the discrete step except at the clamps of Table 1 (eps = 0 or 1,
  * sum eps = 1), where the one-sided derivative inside the unclamped region is used.

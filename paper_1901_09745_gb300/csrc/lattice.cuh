@@ -45,11 +45,11 @@ struct D3Q19 {
 };
 
 // D3Q19 cut into tiles 64 cells wide, for FP32, where one row of 64 cells per warp reads 7 % fewer
-// lines than two of 32 (fewer values beyond a row's ends): 256^3 with 2000 spheres 431 us against
-// 512, without particles 381 against 452. In 2D the narrow tiles are as fast or faster (a disc
-// meets more rows of wide tiles): 2048^2 with 5000 discs 67 us against 70, 777 x 453 19 against
-// 22. wide_tiles tells which lattices take them. Records hold positions from the tile's middle
-// (REC_X), so that they round as finely as with narrow tiles.
+// lines than two of 32 (fewer values beyond a row's ends): 256^3 with 2000 spheres 421 us against
+// 516, without particles 366 against 422. In 2D the narrow tiles are faster (a disc meets more
+// rows of wide tiles: 64 x 4 cells took 1.04 times as long on 2048^2 with 5000 discs, 1.16 times on
+// 777 x 453), so wide ones exist in 3D only. wide_tiles tells which lattices take them. Records hold
+// positions from the tile's middle (REC_X), so that they round as finely as with narrow tiles.
 struct D3Q19w : D3Q19 { static constexpr int TX = 64, TY = 2, TZ = 2, REC_X = 32; };
 
 template <class L>

@@ -94,10 +94,11 @@ __host__ inline long long tile_number(const int dim, const int wide, const Geom 
 }
 // Whether a lattice (g.n and g.faces) is best cut into the wide tiles (D3Q19w in lattice.cuh): FP32
 // in 3D without open faces, where they are at most an eighth of their number emptier than the narrow
-// ones. Step's kernel, narrow and wide, us (tiles wide / narrow): 290 x 128 x 128 200 and 159 (1),
-// 200^3 273 and 231, 198 x 107 x 42 41.2 and 38.6 (1.14), 160 x 128 x 128 80.9 and 84.9 (1.2),
-// 96^3 35.0 and 39.1 (1.33), 32 x 128 x 256 39 and 52 (2), 48^3 15.1 and 15.9 (1): rows of up to 64
-// cells stay narrow, so that a short periodic row needs no minimum image per cell either.
+// ones. A step with a tenth of spheres r = 5, narrow and wide, us (tiles wide / narrow): 290 x 128 x 128
+// 211 and 162 (1), 200^3 286 and 238 (1.14), 198 x 107 x 42 40.3 and 39.2 (1.14), 160 x 128 x 128
+// 82.0 and 87.7 (1.2), 96^3 33.3 and 38.6 (1.33), 32 x 128 x 256 40.6 and 55.7 (2), 48^3 12.2 and 13.9,
+// 64^3 15.9 and 19.7 (1): rows of up to 64 cells stay narrow, so that a short periodic row needs no
+// minimum image per cell either.
 __host__ inline int wide_tiles(const int dim, const size_t elem_bytes, const Geom &g) {
     return elem_bytes == 4 && dim == 3 && g.n[0] > 64 && !open_faces(g) &&
            7 * tile_number(3, 1, g) <= 8 * tile_number(3, 0, g);
@@ -131,7 +132,7 @@ struct Tiles {
     void *blocks;        // per-tile packed candidate records (compute type), see psc_kernels.cuh
     unsigned *order;     // [3 * ntiles] tile numbers: tiles with candidates, then (from ntiles
                          // on) tiles without, then (from 2 ntiles on) tiles with more than
-                         // cap; each list in rising order within a block of 8
+                         // min(cap, kPairCap); each list in rising order within a block of 8
 };
 constexpr int kTileStats = 8;
 constexpr int kCounters = 32, kCounterStride = 32;

@@ -1164,9 +1164,10 @@ cudaError_t launch_step_t(const void *fin, void *fout, const Geom &g, const Phys
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const long long ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
-    // a whole tile per item where every warp of a full chip gets many (256^3: 431 us against 442),
-    // else a unit (2048^2 FP16 64 against 69, 777 x 453 19 against 28); few items go to blocks of
-    // one warp, spread over the SMs
+    // a whole tile per item where every warp of a full chip gets many (256^3 with 2000 spheres, FP32:
+    // 421 us against 456), else a unit (128^3 with 200 62 against 64, 1024^2 FP64 327 against 368,
+    // 777 x 453 15.6 against 24; 2048^2 FP32 65.7 and 65.0); few items go to blocks of one warp,
+    // spread over the SMs
     const int shift = ntiles >= 16LL * 16 * sms ? 0 : 2;
     const long long items = ntiles << shift;
     const int threads = items <= 8LL * sms ? 32 : kPThreads;
@@ -1199,7 +1200,7 @@ cudaError_t launch_fluid_t(const void *fin, void *fout, const Geom &g, const Phy
 
 // One collide-stream step. Without particles: the fluid kernel over every tile. With
 // particles: one kernel over the tiles with candidates and then those without, and the
-// overflow kernel. In a coupled step (ov->defer; 2D, FP32 and 16-bit storage) the tiles with
+// overflow kernel. In a coupled step (ov->defer; 2D FP32) the tiles with
 // candidates and the overflow tiles first, then those without on the second stream, a few
 // blocks per SM, beside the caller's next kernels.
 template <class L, typename S, int PSC, bool VEC>

@@ -23,9 +23,9 @@
 // 16-bit values by such rows takes 350 us, of 32-bit values 376 us; hence rows of 64 cells
 // in 3D. Warps share nothing (no block barrier), so plain-fluid and particle rows interleave
 // freely. Collide-stream kernels of a step, before (two rows of 32 cells, one cell per lane and
-// row, blocks with a barrier per tile) and now, FP32: 256^3 with 2000 spheres 566 -> 431 us, 128^3
-// with 200 spheres 78 -> 66, 2048^2 with 5000 discs 68.7 -> 67, 777 x 453 with 500 discs 20.3 -> 18.5
-// (the state read and written once takes 376, 47, 44 and 3.7 us).
+// row, blocks with a barrier per tile) and now, FP32: 256^3 with 2000 spheres 562 -> 421 us, 128^3
+// with 200 spheres 79 -> 62, 2048^2 with 5000 discs in a band 69 -> 63, 777 x 453 with 500 discs
+// 20.3 -> 15.6 (the state read and written once takes 376, 47, 44 and 3.7 us).
 // Measured slower and not kept: rows copied one unit ahead into shared memory by cp.async (the
 // shared memory comes out of the L1 that loads in flight need: with 200 KB of it a plain copy
 // takes 478 us instead of 371); prefetching the next rows into L2 (30 % slower: as many requests
@@ -594,8 +594,8 @@ template <class L> __device__ __forceinline__ void unit_origin(const Geom &g, co
 // nothing waits for, might land after a clearing store of another. Tiles with more than kPairCap
 // candidates are left to k_collide_overflow.
 //
-// Blocks per SM (registers): more or fewer measured slower (3D FP32 with 5 instead of 4: 256^3 with
-// 2000 spheres 567 us against 431, with 3: 541 against 512 on narrow tiles).
+// Blocks per SM (registers): more or fewer measured slower (3D FP32, 256^3 with 2000 spheres: 5
+// instead of 4 took 1.32 times as long, 3 on narrow tiles 1.06 times).
 template <class L, typename S> __host__ __device__ constexpr int step_blocks() {
     return sizeof(S) == 8 ? 2 : (L::D == 2 ? 6 : 4);
 }

@@ -17,9 +17,11 @@
 // Why not k_step: its sums round differently in the last bits of FP32. Where a value is then
 // rounded to 16 bits, a few in ten thousand come out one unit apart, and after some ten steps the
 // rounding of the whole state has nothing in common with the earlier one. It is as accurate
-// (forces on 5563 spheres after 10 steps of 256^3: 3.2e-5 off FP64 both ways) and faster (756 ->
-// 500 us), but a run's 16-bit results would not be those it gave before. (The adjoint in FP32:
-// see launch_collide_stream_l.)
+// (forces on 5563 spheres after 10 steps of 256^3: 3.2e-5 off FP64 both ways) and faster (748 ->
+// 500 us), but a run's 16-bit results would not be those it gave before. That bears on the order of
+// the sums and of the collision's terms only: k_step's pairs of x-neighbours, its rows of 64 cells
+// and its warps without a barrier would leave a cell's operations as they are. (The adjoint in
+// FP32: see launch_collide_stream_l.)
 
 namespace h16 {
 

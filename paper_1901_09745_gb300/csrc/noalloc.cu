@@ -117,7 +117,8 @@ extern "C" lbm_status lbm_psc_step_noalloc(const lbm_params *p, const void *f_in
         if (p->bc[a] == LBM_BC_INFLOW) ph.inflow_axis = a;
 
     // carve the fixed array: counts | stats | flags | lists | tile order | f(r) | packed tile
-    // blocks; sized for narrow tiles
+    // blocks; sized for narrow tiles (and the order for entries of 8 bytes, twice what it takes, so
+    // that what fits does not depend on either)
     const long long ntiles = (long long)g.nt[0] * g.nt[1] * g.nt[2];
     const long long room = tile_number(is2d ? 2 : 3, 0, g);
     const int rec_double = (p->storage == LBM_F64);
